@@ -406,9 +406,9 @@ VCH_WORKLOADS = {
                         M=4, bc="periodic", seed=0, ic="paper"),
 }
 VCH = dict(VCH_WORKLOADS["mixture"])
-# field words moved per point by one vector CH iteration (two components): passes 1-4 of each
-# component read / write 2+2, 4+2, 2+2 and 5+1 fields; each stage's rhs inverses 4 x (1+1) per component
-VCH_WORDS_ITER, VCH_WORDS_RHS = 40, 16
+# field words moved per point by one vector CH iteration (two components): the nested column and row
+# pass of each component read / write 3+3 and 4+1 fields; each stage's rhs inverses 2 x (1+1) per component
+VCH_WORDS_ITER, VCH_WORDS_RHS = 22, 8
 VCH_SWEEPS_ITER, VCH_SWEEPS_RHS = 14, 8
 # (read, write) fields per point of each vector CH kernel slot; the vector passes 1 and 2 read
 # both components (the column aggregate of pass 1 reads them once more)
@@ -416,6 +416,7 @@ VCH_KERNEL_FIELDS = {
     "rows_H": (1, 1), "rows_pass2": (4, 2), "rows_pass4": (5, 1),
     "cols_agg_H": (1, 0), "cols_agg_pass1": (2, 0), "cols_agg_pass3": (2, 0),
     "cols_final_H": (1, 1), "cols_final_pass1": (2, 2), "cols_final_pass3": (2, 2),
+    "cols_nested": (3, 3), "rows_nested": (4, 1), "cols_nested_rhs": (1, 1), "rows_nested_rhs": (1, 1),
 }
 
 

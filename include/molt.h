@@ -555,7 +555,9 @@ molt_status molt_profile_enable(molt_solver* solver, int enable);
  * summed device milliseconds and launch counts since the last collect; then forget them.
  * Slots: row kernel of fused pass k = k, column aggregate kernel of pass k = 8 + k, column
  * carry kernel = 16, column final kernel of pass k = 17 + k, with k = 0 plain H_c, 1 pass 1,
- * 2 pass 2, 3 pass 3, 4 pass 4, 5 and 6 the two 1D passes. */
+ * 2 pass 2, 3 pass 3, 4 pass 4, 5 and 6 the two 1D passes.  Nested passes of the 2D iteration
+ * with equal factors (two inverses per axis in one kernel): rows = 7, columns = 24, and 15 / 25 for
+ * the inverse of a stage's right side. */
 #define MOLT_PROFILE_SLOTS 32
 molt_status molt_profile_collect(molt_solver* solver, double* ms, long long* launches);
 

@@ -156,6 +156,46 @@ cudaError_t sweep(int axis, const LineParams<T>& lp, int kind, const OpArgs<T>& 
                   ColScratch<T>* cs, unsigned long long* red, cudaStream_t st, long long* launches,
                   Prof* prof = nullptr);
 
+// ---- nested passes (nest.cuh, nest_rows.cuh): two inverses of one c along an axis in one pass ----
+// profile slots: the iteration's passes, the rhs inverse
+constexpr int kProfNestRows = 7, kProfNestCols = 24, kProfNestRowsRhs = 15, kProfNestColsRhs = 25;
+// What a nested column pass computes (nest.cuh).
+enum NestColMode { NEST_SCALAR = 0, NEST_VCH = 1, NEST_Z3 = 2, NEST_COPY = 3 };
+enum NestRowMode { NEST_ROW_PASS = 0, NEST_ROW_COPY = 1 };
+template <typename T>
+struct NestCols {
+    const T *in0 = nullptr, *in1 = nullptr, *Y = nullptr;
+    T *o0 = nullptr, *o1 = nullptr, *o2 = nullptr;
+    long long ld = 0, slab = 0;    // distances of two nodes of a column and of two slabs of columns
+    int ncols = 0, nslabs = 1;
+    T g1 = 0, beta = 0, vs = 0;
+    int comp = 0;
+};
+template <typename T>
+struct NestRows {
+    const T *A = nullptr, *B = nullptr, *E = nullptr;
+    T* w = nullptr;
+    int nlines = 0, fix = 0;
+    T wall = 0;
+    unsigned long long* red = nullptr;
+};
+// Whether the nested passes take lines of n nodes along rows / columns.
+template <typename T>
+bool nest_rows_ok(int n);
+template <typename T>
+bool nest_cols_ok(int n);
+template <typename T>
+cudaError_t nest_cols(const LineParams<T>& lp, int mode, const NestCols<T>& p, cudaStream_t st, long long* launches,
+                      Prof* prof = nullptr);
+template <typename T>
+cudaError_t nest_rows(const LineParams<T>& lp, int mode, const NestRows<T>& p, cudaStream_t st, long long* launches,
+                      Prof* prof = nullptr);
+// ... of one quadrature order (one translation unit each)
+template <int M, typename T>
+cudaError_t nest_cols_m(const LineParams<T>& lp, int mode, const NestCols<T>& p, cudaStream_t st, Prof* prof);
+template <int M, typename T>
+cudaError_t nest_rows_m(const LineParams<T>& lp, int mode, const NestRows<T>& p, cudaStream_t st, Prof* prof);
+
 // Largest line length the row kernel supports for a field count (shared-memory bound).
 template <typename T>
 int max_row_length(int nf);

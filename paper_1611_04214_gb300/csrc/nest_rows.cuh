@@ -1,0 +1,410 @@
+// Two line inverses in a row along x (rows), the line in registers between them (see nest.cuh).
+// A team of TL threads owns a line: thread t holds chunk t, and in packed FP32 chunk t of the
+// line's first half in the low and of its second half in the high half of each register pair.  Teams of
+// up to 32 threads are parts of a warp (no block barrier anywhere), longer lines take a block.
+//   pass:  w <- w + (E + H (B + H A)), with the residual of the iteration (E = Y - H_y H_y w);
+//   copy:  out = H H in.
+// Bound: the latency of a line's chain (load, two scans, loads of B, E and w) at two lines a SM: 8192^2 FP32 285 us
+// = 4700 GB/s of its 20 B a point (0.69 of the copy rate) for two inverses, against 306 + 237 us of passes 2 and 4; the
+// fetches into L2 ahead of use give 5% of it.
+#pragma once
+
+#include "nest.cuh"
+
+namespace molt {
+
+template <typename T>
+struct NestRowArgs {
+    const T* A;
+    const T* B;
+    const T* E;
+    T* w;            // pass: the iterate, in place; copy: the output
+    int nlines;
+    int half;        // nodes of a register half (n or n / 2)
+    int TL;          // threads per line
+    NestCut cut;     // of a half
+    int fix;         // Dirichlet grids: write `wall` to the wall nodes
+    T wall;
+    unsigned long long* red;
+    NestPow<T> pw;   // d^(cnt-1) of the two chunk lengths
+    int ahead;       // lines resident at a time (0: nothing is fetched ahead)
+};
+
+template <class N>
+struct NestRowShared {
+    using V = typename N::V;
+    using T = typename N::T;
+    V tot[2][16];
+    V ex[2][16];
+    V X[2];
+    T wd[16], wdf[16], wdb[16];
+};
+
+template <typename T>
+struct NestRowScan {
+    int lane, warp, nwarps, tl, width;
+    T df[5], db[5];
+    T Dxf, Dxb;      // decay of the scan group's chunks before / after this one
+    T Dh;            // decay over a half
+    T pl[2], pr[2];  // decay from the line's ends, per half
+};
+
+// Totals of the halves -> carries entering the halves (E) and line totals.
+template <class N>
+__device__ __forceinline__ void nest_halves(typename N::V f, typename N::V b, typename N::T Dh, typename N::V& Ef,
+                                            typename N::V& Eb, typename N::T& IN, typename N::T& I0) {
+    using T = typename N::T;
+    if constexpr (N::W == 2) {
+        Ef = N::pair(T(0), N::get(f, 0));
+        Eb = N::pair(N::get(b, 1), T(0));
+        IN = ::fma(N::get(f, 0), Dh, N::get(f, 1));
+        I0 = ::fma(N::get(b, 1), Dh, N::get(b, 0));
+    } else {
+        Ef = Eb = N::zero();
+        IN = f;
+        I0 = b;
+    }
+}
+
+template <class N, bool WARP>
+__device__ __forceinline__ void nest_row_scan(const LineParams<typename N::T>& lp, const NestRowScan<typename N::T>& c,
+                                              NestRowShared<N>& sh, typename N::V aL, typename N::V aR,
+                                              typename N::V& cL, typename N::V& cR, typename N::V& XL,
+                                              typename N::V& XR) {
+    using V = typename N::V;
+    using T = typename N::T;
+    V a = aL, b = aR;
+    const int width = WARP ? c.width : 32, li = c.lane & (width - 1);
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+        const int o = 1 << s;
+        if (o < width) {
+            const V u = shfl_up_v<N>(a, o, width), v = shfl_down_v<N>(b, o, width);
+            if (li >= o) a = N::fma(u, N::splat(c.df[s]), a);
+            if (li + o < width) b = N::fma(v, N::splat(c.db[s]), b);
+        }
+    }
+    V ax = shfl_up_v<N>(a, 1, width), bx = shfl_down_v<N>(b, 1, width);
+    if (li == 0) ax = N::zero();
+    if (li == width - 1) bx = N::zero();
+    V Ef, Eb;
+    T IN, I0, xl, xr;
+    if constexpr (WARP) {
+        const V f = __shfl_sync(kFull, a, width - 1, width), g = __shfl_sync(kFull, b, 0, width);
+        nest_halves<N>(f, g, c.Dh, Ef, Eb, IN, I0);
+        nest_boundary<T>(lp, I0, IN, xl, xr);
+        XL = N::splat(xl);
+        XR = N::splat(xr);
+    } else {
+        if (c.lane == 31) sh.tot[0][c.warp] = a;
+        if (c.lane == 0) sh.tot[1][c.warp] = b;
+        __syncthreads();
+        if (c.warp == 0) {
+            // scan of the warps' totals, one warp per lane
+            const bool has = c.lane < c.nwarps;
+            V f = has ? sh.tot[0][c.lane] : N::zero(), g = has ? sh.tot[1][c.lane] : N::zero();
+            T fd = has ? sh.wd[c.lane] : T(1), gd = fd;
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) {
+                const V u = shfl_up_v<N>(f, o), v = shfl_down_v<N>(g, o);
+                const T ud = __shfl_up_sync(kFull, fd, o), vd = __shfl_down_sync(kFull, gd, o);
+                if (c.lane >= o) {
+                    f = N::fma(u, N::splat(fd), f);
+                    fd *= ud;
+                }
+                if (c.lane + o < 32) {
+                    g = N::fma(v, N::splat(gd), g);
+                    gd *= vd;
+                }
+            }
+            const V tf = __shfl_sync(kFull, f, c.nwarps - 1), tg = __shfl_sync(kFull, g, 0);
+            V fx = shfl_up_v<N>(f, 1), gx = shfl_down_v<N>(g, 1);
+            if (c.lane == 0) fx = N::zero();
+            if (c.lane >= c.nwarps - 1) gx = N::zero();
+            nest_halves<N>(tf, tg, c.Dh, Ef, Eb, IN, I0);
+            nest_boundary<T>(lp, I0, IN, xl, xr);
+            if (has) {
+                sh.ex[0][c.lane] = N::fma(Ef, N::splat(sh.wdf[c.lane]), fx);
+                sh.ex[1][c.lane] = N::fma(Eb, N::splat(sh.wdb[c.lane]), gx);
+            }
+            if (c.lane == 0) {
+                sh.X[0] = N::splat(xl);
+                sh.X[1] = N::splat(xr);
+            }
+        }
+        __syncthreads();
+        Ef = sh.ex[0][c.warp];
+        Eb = sh.ex[1][c.warp];
+        XL = sh.X[0];
+        XR = sh.X[1];
+    }
+    const V pl = N::pair(c.pl[0], c.pl[1]), pr = N::pair(c.pr[0], c.pr[1]);
+    cL = N::fma(pl, XL, N::fma(Ef, N::splat(c.Dxf), ax));
+    cR = N::fma(pr, XR, N::fma(Eb, N::splat(c.Dxb), bx));
+}
+
+// Edge values of the neighbouring chunks of the line (wrapped; a low half continues in the high half).
+template <class N, int K, int M, int S, bool RAG, bool WARP, int KM>
+__device__ __forceinline__ void nest_row_halo(const NestRowScan<typename N::T>& c, int nc, int cnt,
+                                              typename N::V* edge, int TL, typename N::V (&x)[KM]) {
+    using V = typename N::V;
+    constexpr int H = M / 2;
+    V l[H], r[H];
+    const int tl = c.tl;
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        V e = x[H + K - H + h];
+        if (RAG && cnt != K) e = x[H + K - S - H + h];
+        if constexpr (WARP) {
+            const int base = c.lane - tl;
+            const int pl = base + (tl > 0 ? tl - 1 : nc - 1), fl = base + (tl < nc - 1 ? tl + 1 : 0);
+            l[h] = __shfl_sync(kFull, e, pl);
+            r[h] = __shfl_sync(kFull, x[H + h], fl);
+        } else {
+            edge[h * TL + tl] = e;
+            edge[(H + h) * TL + tl] = x[H + h];
+        }
+    }
+    if constexpr (!WARP) {
+        __syncthreads();
+        const int pl = tl > 0 ? tl - 1 : nc - 1, fl = tl < nc - 1 ? tl + 1 : 0;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            l[h] = edge[h * TL + pl];
+            r[h] = edge[(H + h) * TL + fl];
+        }
+    }
+    if constexpr (N::W == 2) {
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            if (tl == 0) l[h] = N::swap(l[h]);
+            if (tl == nc - 1) r[h] = N::swap(r[h]);
+        }
+    }
+    nest_set_halo<N, K, M, S, RAG>(cnt, l, r, x);
+}
+
+// Nodes p.. of one half line (float4 chunks), or of a scalar line.
+template <class N, int K, bool RAG, int OFF, int KM>
+__device__ __forceinline__ void nest_row_load(const typename N::T* f, int half, int start, int cnt, bool on,
+                                              typename N::V (&x)[KM]) {
+    using T = typename N::T;
+    if constexpr (N::W == 2) {
+#pragma unroll
+        for (int j = 0; j < K / 4; ++j) {
+            float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+            if (on && (!RAG || 4 * j < cnt)) {
+                lo = *reinterpret_cast<const float4*>(f + start + 4 * j);
+                hi = *reinterpret_cast<const float4*>(f + half + start + 4 * j);
+            }
+            x[OFF + 4 * j] = N::pair(lo.x, hi.x);
+            x[OFF + 4 * j + 1] = N::pair(lo.y, hi.y);
+            x[OFF + 4 * j + 2] = N::pair(lo.z, hi.z);
+            x[OFF + 4 * j + 3] = N::pair(lo.w, hi.w);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < K; ++k) x[OFF + k] = on && (!RAG || k < cnt) ? f[start + k] : T(0);
+    }
+}
+
+// Block maximum of the residual values into the FP64 slots; blocks that would not raise a slot leave
+// it alone (the slots only grow, so a stale read costs an atomic at most).
+template <typename T>
+__device__ __forceinline__ T nest_warp_max(T v) {
+    if constexpr (sizeof(T) == 4) {
+        // non-negative floats order like their bits
+        return __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(v)));
+    } else {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
+        return v;
+    }
+}
+template <typename T>
+__device__ __forceinline__ void nest_reduce(RedAcc<T> r, unsigned long long* slots) {
+    __shared__ T s_max[2][16];
+    const T dm = nest_warp_max(r.dmax), vm = nest_warp_max(r.vmax);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (lane == 0) {
+        s_max[0][warp] = dm;
+        s_max[1][warp] = vm;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        T m = T(0);
+        for (int w = 0; w < nw; ++w) m = fmax(m, s_max[threadIdx.x][w]);
+        const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(static_cast<double>(m)));
+        if (b > *static_cast<volatile unsigned long long*>(slots + threadIdx.x)) atomicMax(slots + threadIdx.x, b);
+    }
+}
+
+template <class N, int M, bool RAG, bool WARP, int MODE>
+__global__ void __launch_bounds__(N::W == 2 ? 256 : 512, N::W == 2 ? 2 : 1)
+nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
+                 const __grid_constant__ NestCoef<typename N::V> w,
+                 const __grid_constant__ NestRowArgs<typename N::T> a) {
+    using V = typename N::V;
+    using T = typename N::T;
+    constexpr int K = kNestRowK, H = M / 2, S = 1;
+    extern __shared__ __align__(16) unsigned char nest_row_sm[];
+    V* edge = reinterpret_cast<V*>(nest_row_sm);      // two sets of 2 H values per thread (block teams)
+    __shared__ NestRowShared<N> sh;
+    NestRowScan<T> c;
+    c.lane = threadIdx.x & 31;
+    c.warp = threadIdx.x >> 5;
+    c.nwarps = blockDim.x >> 5;
+    c.width = a.TL < 32 ? a.TL : 32;
+    int line;
+    if constexpr (WARP) {
+        c.tl = c.lane & (a.TL - 1);
+        line = (blockIdx.x * c.nwarps + c.warp) * (32 / a.TL) + c.lane / a.TL;
+    } else {
+        c.tl = threadIdx.x;
+        line = blockIdx.x;
+    }
+    const bool live = c.tl < a.cut.nc, on = live && line < a.nlines;
+    const int ci = live ? c.tl : 0;
+    NestChunk ck;
+    ck.cnt = !live ? 0 : (!RAG || ci < a.cut.rem) ? K : K - S;
+    const int start = RAG ? ci * (K - S) + S * min(ci, a.cut.rem) : ci * K;
+    const bool periodic = lp.bc == BC_PERIODIC;
+    ck.mA = live && !periodic && ci == 0 ? 1 : 0;
+    ck.mB = live && !periodic && ci == a.cut.nc - 1 ? N::W : 0;
+    const size_t row = static_cast<size_t>(on ? line : 0) * lp.n;
+
+    V x[K + M];
+    nest_row_load<N, K, RAG, H>(a.A + row, a.half, start, ck.cnt, on, x);
+    if (a.ahead) {
+        // the fields that this line needs later, and the first one of the line after the resident ones, into L2
+        const int step = 128 / sizeof(T);
+        const size_t next = static_cast<size_t>(line + a.ahead < a.nlines ? line + a.ahead : a.nlines - 1) * lp.n;
+        for (int p = c.tl * step; p < lp.n; p += a.TL * step) {
+            if constexpr (MODE == NEST_ROW_PASS) {
+                nest_prefetch(a.B + row + p);
+                nest_prefetch(a.E + row + p);
+                nest_prefetch(a.w + row + p);
+            }
+            nest_prefetch(a.A + next + p);
+        }
+    }
+
+    // ---- scan constants ----
+    {
+        const T D = ck.cnt == 0 ? T(1) : (!RAG || ck.cnt == K) ? a.pw.full * lp.d : a.pw.less * lp.d;
+        T f = D, b = D;
+        const int li = c.lane & (c.width - 1);
+#pragma unroll
+        for (int s = 0; s < 5; ++s) {
+            const int o = 1 << s;
+            c.df[s] = f;
+            c.db[s] = b;
+            if (o < c.width) {
+                const T u = __shfl_up_sync(kFull, f, o, c.width), v = __shfl_down_sync(kFull, b, o, c.width);
+                if (li >= o) f *= u;
+                if (li + o < c.width) b *= v;
+            }
+        }
+        c.Dxf = __shfl_up_sync(kFull, f, 1, c.width);
+        c.Dxb = __shfl_down_sync(kFull, b, 1, c.width);
+        if (li == 0) c.Dxf = T(1);
+        if (li == c.width - 1) c.Dxb = T(1);
+        c.Dh = dev_exp(-lp.nu * T(a.half));
+        const int last = start + ck.cnt;
+#pragma unroll
+        for (int q = 0; q < N::W; ++q) {
+            const int p = q * a.half, m = periodic ? 0 : 1;   // a wall's value starts one node later
+            c.pl[q] = dev_exp(-lp.nu * T(max(p + start - m, 0)));
+            c.pr[q] = dev_exp(-lp.nu * T(max(lp.n - p - last - m, 0)));
+        }
+        if constexpr (N::W == 1) c.pl[1] = c.pr[1] = T(0);
+        if constexpr (!WARP) {
+            if (c.lane == 31) sh.wd[c.warp] = f;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                T p = T(1);
+                for (int w = 0; w < c.nwarps; ++w) {
+                    sh.wdf[w] = p;
+                    p *= sh.wd[w];
+                }
+                p = T(1);
+                for (int w = c.nwarps - 1; w >= 0; --w) {
+                    sh.wdb[w] = p;
+                    p *= sh.wd[w];
+                }
+            }
+        }
+    }
+    const T d = lp.d;
+    V aL, aR, cL, cR, XL, XR, out[K];
+    nest_row_halo<N, K, M, S, RAG, WARP>(c, a.cut.nc, ck.cnt, edge, a.TL, x);
+    nest_chunk_agg<N, K, M, S, RAG>(w, d, a.pw, ck, x, aL, aR);
+    nest_row_scan<N, WARP>(lp, c, sh, aL, aR, cL, cR, XL, XR);
+    nest_chunk_finish<N, K, M, S, RAG>(w, d, ck, x, cL, cR, [&](int dir) { return dir ? XR : XL; }, out);
+    if constexpr (MODE == NEST_ROW_PASS) nest_row_load<N, K, RAG, H>(a.B + row, a.half, start, ck.cnt, on, x);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if constexpr (MODE == NEST_ROW_PASS) x[H + k] = N::add(x[H + k], out[k]);
+        else x[H + k] = out[k];
+    }
+    nest_row_halo<N, K, M, S, RAG, WARP>(c, a.cut.nc, ck.cnt, edge + 2 * H * a.TL, a.TL, x);
+    nest_chunk_agg<N, K, M, S, RAG>(w, d, a.pw, ck, x, aL, aR);
+    nest_row_scan<N, WARP>(lp, c, sh, aL, aR, cL, cR, XL, XR);
+    nest_chunk_finish<N, K, M, S, RAG>(w, d, ck, x, cL, cR, [&](int dir) { return dir ? XR : XL; }, out);
+
+    if constexpr (MODE == NEST_ROW_COPY) {
+        if constexpr (N::W == 2) {
+#pragma unroll
+            for (int j = 0; j < K / 4; ++j)
+                if (on && (!RAG || 4 * j < ck.cnt)) {
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        *reinterpret_cast<float4*>(a.w + row + q * a.half + start + 4 * j) =
+                            make_float4(N::get(out[4 * j], q), N::get(out[4 * j + 1], q), N::get(out[4 * j + 2], q),
+                                        N::get(out[4 * j + 3], q));
+                }
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (on && (!RAG || k < ck.cnt)) a.w[row + start + k] = out[k];
+        }
+    } else {
+        RedAcc<T> red{T(0), T(0)};
+        const bool wall_row = a.fix && (line == 0 || line == a.nlines - 1);
+        auto put = [&](T h, T e, T o, int p) {
+            const T nw = o + (e + h);
+            red.dmax = fmax(red.dmax, fabs(nw - o));
+            red.vmax = fmax(red.vmax, fabs(nw));
+            return a.fix && (wall_row || p == 0 || p == lp.n - 1) ? a.wall : nw;
+        };
+        if constexpr (N::W == 2) {
+#pragma unroll
+            for (int j = 0; j < K / 4; ++j)
+                if (on && (!RAG || 4 * j < ck.cnt)) {
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int p = q * a.half + start + 4 * j;
+                        const float4 e = *reinterpret_cast<const float4*>(a.E + row + p);
+                        float4* dst = reinterpret_cast<float4*>(a.w + row + p);
+                        const float4 o = *dst;
+                        float4 v;
+                        v.x = put(N::get(out[4 * j], q), e.x, o.x, p);
+                        v.y = put(N::get(out[4 * j + 1], q), e.y, o.y, p + 1);
+                        v.z = put(N::get(out[4 * j + 2], q), e.z, o.z, p + 2);
+                        v.w = put(N::get(out[4 * j + 3], q), e.w, o.w, p + 3);
+                        *dst = v;
+                    }
+                }
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (on && (!RAG || k < ck.cnt)) {
+                    const size_t i = row + start + k;
+                    a.w[i] = put(out[k], a.E[i], a.w[i], start + k);
+                }
+        }
+        nest_reduce<T>(red, a.red);
+    }
+}
+
+}  // namespace molt

@@ -18,6 +18,11 @@
 //        (x, c_o)  w <- Y + w - Q2 + H_ox(Q1 - U)
 //   which is, term by term, Y + M_o^{-1}[beta (M_i^{-1}G - G + D_ix D_iy G)]
 //   + (D_ox D_oy + D_ix D_iy - D_ox D_oy D_ix D_iy) w  (Sec. 5.1 with c_o != c_i).
+//   Equal factors (c_o = c_i, the completed square): the x and y inverses commute, so the same
+//   map collects into one pass per axis with two inverses each (nest.cuh),
+//        (y)  s = H_y w,  b = H_y G,  t = H_y s,  a = H_y b,
+//             A = beta (2a - b) - w + 2s - t,  B = -beta a - 2 (s - t),  E = Y - t
+//        (x)  w <- w + E + H_x (B + H_x A).
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -454,6 +459,24 @@ struct Solver final : molt_solver {
         return copy_sweep(0, lx, f1, out, st, c);
     }
 
+    // out = M_{c_out}^{-1} M_{c_in}^{-1} in: one nested pass per axis for equal factors, four sweeps
+    // otherwise (scratch f1, f2).
+    cudaError_t rhs_inverse(double c_in, double c_out, const T* in, T* out, cudaStream_t st, bool vch = false) {
+        cudaError_t e;
+        if (use_nest(c_in, c_out, vch)) {
+            molt::LineParams<T> lx, ly;
+            if (!line_params(c_in, 0, &lx) || !line_params(c_in, 1, &ly)) return cudaErrorInvalidValue;
+            molt::NestCols<T> c;
+            c.in0 = in, c.o0 = f1, c.ld = g.nx, c.ncols = g.nx;
+            if ((e = molt::nest_cols<T>(ly, molt::NEST_COPY, c, st, &launches, &prof)) != cudaSuccess) return e;
+            molt::NestRows<T> r;
+            r.A = f1, r.w = out, r.nlines = g.ny;
+            return molt::nest_rows<T>(lx, molt::NEST_ROW_COPY, r, st, &launches, &prof);
+        }
+        if ((e = mm_inv(c_in, in, f2, st)) != cudaSuccess) return e;
+        return mm_inv(c_out, f2, out, st);
+    }
+
     // out = E_c in with E = M^{-1} - I + D_x D_y, i.e. 2 H_x H_y - H_x - H_y in 2D and H - I in 1D
     // (the operator through which M^{-1} acts on c Lap, Remark Laplacian); scratch f1, f2, f3.
     cudaError_t e_op(double c, const T* in, T* out, cudaStream_t st) {
@@ -519,8 +542,44 @@ struct Solver final : molt_solver {
         T g2, g1, beta, s;
         bool two_d;
         bool vch = false;   // vector CH iteration (both components)
+        bool nest = false;  // equal factors: one column and one row pass (see the file comment)
         T vs = 0;           // vector CH: (c1 + c2)/tau
     };
+
+    // Whether the nested passes run a 2D iteration with equal factors (us per iteration, the four passes
+    // against the nested ones, M = 4):
+    //   FP64: every size (1024^2 510 / 309, 2048^2 1777 / 1072).
+    //   FP32: from 256 nodes a side (shorter lines run the block bodies of the batched path, which the
+    //   single grid matches bit for bit); 1024^2 periodic / Neumann 46 / 25 and 60 / 28, 2048^2 92 / 82 and
+    //   128 / 83, 3000 x 2000 276 / 163.  Columns of more than 2048 nodes are spread over clusters of 8 or 16
+    //   blocks whose exchanges cost what the saved traffic gives: 4096^2 Neumann 318 / 292 but periodic
+    //   282 / 295, 2048 x 8192 276 / 332; so there only the grids that the pipelined kernels of the four
+    //   passes serve badly (walls, unaligned lines) and the vector model (767 / 660) take them, up to 4096.
+    bool use_nest(double c_in, double c_out, bool vch = false) const {
+        if (g.dim != 2 || c_in != c_out) return false;
+        if (fp32()) {
+            if (g.nx < 256 || g.ny < 256 || g.ny > 4096) return false;
+            if (g.ny > 2048 && !vch && bc == molt::BC_PERIODIC && g.nx % 512 == 0) return false;
+        }
+        return molt::nest_rows_ok<T>(g.nx) && molt::nest_cols_ok<T>(g.ny);
+    }
+
+    // The column pass of one field (or component) and the row pass that completes the iterate.
+    cudaError_t nest_columns(const Passes& ps, const T* in0, const T* in1, const T* y, T* A, T* B, T* E, int comp,
+                             cudaStream_t st) {
+        molt::NestCols<T> c;
+        c.in0 = in0, c.in1 = in1, c.Y = y, c.o0 = A, c.o1 = B, c.o2 = E;
+        c.ld = g.nx, c.ncols = g.nx;
+        c.g1 = ps.g1, c.beta = ps.beta, c.vs = ps.vs, c.comp = comp;
+        return molt::nest_cols<T>(ps.liy, ps.vch ? molt::NEST_VCH : molt::NEST_SCALAR, c, st, &launches, &prof);
+    }
+    cudaError_t nest_row_pass(const Passes& ps, const T* A, const T* B, const T* E, T* field, double wall,
+                              cudaStream_t st) {
+        molt::NestRows<T> r;
+        r.A = A, r.B = B, r.E = E, r.w = field, r.nlines = g.ny, r.red = red;
+        r.fix = bc == molt::BC_DIRICHLET, r.wall = static_cast<T>(wall);
+        return molt::nest_rows<T>(ps.lix, molt::NEST_ROW_PASS, r, st, &launches, &prof);
+    }
 
     bool make_passes(const StageParams& sp, Passes* ps) {
         ps->two_d = g.dim == 2;
@@ -530,6 +589,7 @@ struct Solver final : molt_solver {
         ps->g2 = ps->s == T(1) ? T(0) : T(-3);
         ps->g1 = ps->s == T(1) ? static_cast<T>(sp.lam - 3.0) : static_cast<T>(sp.lam);
         ps->beta = static_cast<T>(sp.beta);
+        ps->nest = use_nest(sp.c_in, sp.c_out);
         return true;
     }
 
@@ -555,6 +615,7 @@ struct Solver final : molt_solver {
         ps->g2 = ps->g1 = T(0);
         ps->beta = static_cast<T>(tau / *c_in);
         ps->vch = true;
+        ps->nest = use_nest(*c_in, *c_out, true);
         ps->vs = static_cast<T>((c1 + c2) / tau);
         return true;
     }
@@ -567,6 +628,16 @@ struct Solver final : molt_solver {
         T* V[2] = {w, vw2};
         const T* Yc[2] = {Y, vY2};
         if (ps.two_d) {
+            if (ps.nest) {
+                T* A[2] = {f1, f4};
+                T* B[2] = {f2, f5};
+                T* E[2] = {f3, f6};
+                for (int c = 0; c < 2; ++c)
+                    if ((e = nest_columns(ps, w, vw2, Yc[c], A[c], B[c], E[c], c, st)) != cudaSuccess) return e;
+                for (int c = 0; c < 2; ++c)
+                    if ((e = nest_row_pass(ps, A[c], B[c], E[c], V[c], 0.0, st)) != cudaSuccess) return e;
+                return cudaSuccess;
+            }
             T* U[2] = {f4, vg4};
             T* Q1[2] = {f5, vg5};
             T* Q2[2] = {f6, vg6};
@@ -618,6 +689,10 @@ struct Solver final : molt_solver {
     cudaError_t launch_iteration(const Passes& ps, cudaStream_t st) {
         if (ps.vch) return launch_vch_iteration(ps, st);
         cudaError_t e;
+        if (ps.nest) {
+            if ((e = nest_columns(ps, w, nullptr, Y, f1, f2, f3, 0, st)) != cudaSuccess) return e;
+            return nest_row_pass(ps, f1, f2, f3, w, -1.0, st);
+        }
         if (ps.two_d) {
             // Block orders alternate so that each pass starts at the end of the field the pass
             // before it finished on (still in L2): pass 4 ends at the last row, pass 1 aggregates
@@ -738,8 +813,7 @@ struct Solver final : molt_solver {
         cudaError_t e = cudaSuccess;
         if (!y_given) {
             // Y = M_o^{-1} M_i^{-1} r
-            if ((e = mm_inv(sp.c_in, rhs, f2, st)) != cudaSuccess) return cuda_fail(e, "rhs inverse");
-            if ((e = mm_inv(sp.c_out, f2, Y, st)) != cudaSuccess) return cuda_fail(e, "rhs inverse");
+            if ((e = rhs_inverse(sp.c_in, sp.c_out, rhs, Y, st)) != cudaSuccess) return cuda_fail(e, "rhs inverse");
         }
         if (!given && bc == molt::BC_DIRICHLET && (e = add_dirichlet_offset(sp, Y, st)) != cudaSuccess)
             return cuda_fail(e, "Dirichlet offset");
@@ -872,13 +946,13 @@ struct Solver final : molt_solver {
             return cuda_fail(e, "sdc state");                                  // v0_{n+1}
         if (start) {
             if ((e = lin(r, wn, 1.0, k0, -0.5 * dt, nullptr, 0, nullptr, 0, 0, st)) != cudaSuccess ||
-                (e = mm_inv(sp.c_in, r, f2, st)) != cudaSuccess || (e = mm_inv(sp.c_out, f2, Y, st)) != cudaSuccess ||
+                (e = rhs_inverse(sp.c_in, sp.c_out, r, Y, st)) != cudaSuccess ||
                 (e = inverse_of_F(sp, v0n, sdc_F0, st)) != cudaSuccess ||
                 (e = lin(Y, Y, 1.0, sdc_F0, 0.5 * dt, nullptr, 0, nullptr, 0, 0, st)) != cudaSuccess)
                 return cuda_fail(e, "sdc rhs");
         } else {
             if ((e = lin(r, wn, 1.0, k0, -0.5 * dt, sdc_F0, 0.5 * dt, nullptr, 0, 0, st)) != cudaSuccess ||
-                (e = mm_inv(sp.c_in, r, f2, st)) != cudaSuccess || (e = mm_inv(sp.c_out, f2, Y, st)) != cudaSuccess)
+                (e = rhs_inverse(sp.c_in, sp.c_out, r, Y, st)) != cudaSuccess)
                 return cuda_fail(e, "sdc rhs");
         }
         ms = stage(dt, nullptr, st, &it, &res, &tu, true);                     // level [1]
@@ -1143,8 +1217,8 @@ struct Solver final : molt_solver {
         Passes ps;
         double c_in, c_out;
         if (!make_vch_passes(tau, &ps, &c_in, &c_out)) return MOLT_ERR_ARG;
-        if ((e = mm_inv(c_in, r1, f2, st)) != cudaSuccess || (e = mm_inv(c_out, f2, Y, st)) != cudaSuccess ||
-            (e = mm_inv(c_in, r2, f2, st)) != cudaSuccess || (e = mm_inv(c_out, f2, vY2, st)) != cudaSuccess)
+        if ((e = rhs_inverse(c_in, c_out, r1, Y, st, true)) != cudaSuccess ||
+            (e = rhs_inverse(c_in, c_out, r2, vY2, st, true)) != cudaSuccess)
             return cuda_fail(e, "vector CH rhs inverse");
         int it;
         double res, tu;
@@ -1181,8 +1255,8 @@ struct Solver final : molt_solver {
         Passes ps;
         double c_in, c_out;
         if (!make_vch_passes(tau, &ps, &c_in, &c_out)) return MOLT_ERR_ARG;
-        if ((e = mm_inv(c_in, r, f2, st)) != cudaSuccess || (e = mm_inv(c_out, f2, Y, st)) != cudaSuccess ||
-            (e = mm_inv(c_in, vr2, f2, st)) != cudaSuccess || (e = mm_inv(c_out, f2, vY2, st)) != cudaSuccess)
+        if ((e = rhs_inverse(c_in, c_out, r, Y, st, true)) != cudaSuccess ||
+            (e = rhs_inverse(c_in, c_out, vr2, vY2, st, true)) != cudaSuccess)
             return cuda_fail(e, "vector stage rhs inverse");
         double res, tu;
         molt_status ms = stage(tau, nullptr, st, iters, &res, &tu, true, &ps);

@@ -37,6 +37,7 @@ EXPORTS = [
 ]
 EXECUTION = {"host_loop": 0, "graph": 1}
 PROFILE_SLOTS = 32
+NESTED_SLOTS = {7: "rows_nested", 15: "rows_nested_rhs", 24: "cols_nested", 25: "cols_nested_rhs"}
 PASS_NAMES = ["H", "pass1", "pass2", "pass3", "pass4", "pass1d_a", "pass1d_b", ""]
 
 
@@ -421,7 +422,9 @@ class Solver:
         for slot in range(PROFILE_SLOTS):
             if cnt[slot] == 0:
                 continue
-            if slot < 8:
+            if slot in NESTED_SLOTS:
+                name = NESTED_SLOTS[slot]
+            elif slot < 8:
                 name = f"rows_{PASS_NAMES[slot]}"
             elif slot < 16:
                 name = f"cols_agg_{PASS_NAMES[slot - 8]}"
