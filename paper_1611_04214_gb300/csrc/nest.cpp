@@ -1,7 +1,23 @@
 // Entry of the nested passes: eligibility and the dispatch on the quadrature order.
+#include <cmath>
+
 #include "nest_shape.h"
 
 namespace molt {
+
+// The line parameters of nu' = -ln d for the decay d as the kernels hold it: recurrence, weights and boundary
+// coefficients then belong to one operator (H 1 = 1 holds with a rounded d too).  They depend on nu alone.
+template <typename T>
+LineParams<T> nest_line_params(const LineParams<T>& lp) {
+    const double d = static_cast<double>(lp.d);
+    LineParams<double> p;
+    const char* err = nullptr;
+    if (sizeof(T) == 8 || !(d > 0.0 && d < 1.0) || !build_line_params(1.0, -std::log(d), lp.n, lp.M, lp.bc, &p, &err))
+        return lp;
+    LineParams<T> q = cast_line_params<T>(p);
+    q.d = lp.d;
+    return q;
+}
 
 template <typename T>
 bool nest_rows_ok(int n) {
@@ -21,10 +37,11 @@ template <typename T>
 cudaError_t nest_cols(const LineParams<T>& lp, int mode, const NestCols<T>& p, cudaStream_t st, long long* launches,
                       Prof* prof) {
     if (launches) *launches += 1;
+    const LineParams<T> q = nest_line_params(lp);
     switch (lp.M) {
-        case 2: return nest_cols_m<2, T>(lp, mode, p, st, prof);
-        case 4: return nest_cols_m<4, T>(lp, mode, p, st, prof);
-        case 6: return nest_cols_m<6, T>(lp, mode, p, st, prof);
+        case 2: return nest_cols_m<2, T>(q, mode, p, st, prof);
+        case 4: return nest_cols_m<4, T>(q, mode, p, st, prof);
+        case 6: return nest_cols_m<6, T>(q, mode, p, st, prof);
     }
     return cudaErrorInvalidValue;
 }
@@ -33,15 +50,17 @@ template <typename T>
 cudaError_t nest_rows(const LineParams<T>& lp, int mode, const NestRows<T>& p, cudaStream_t st, long long* launches,
                       Prof* prof) {
     if (launches) *launches += 1;
+    const LineParams<T> q = nest_line_params(lp);
     switch (lp.M) {
-        case 2: return nest_rows_m<2, T>(lp, mode, p, st, prof);
-        case 4: return nest_rows_m<4, T>(lp, mode, p, st, prof);
-        case 6: return nest_rows_m<6, T>(lp, mode, p, st, prof);
+        case 2: return nest_rows_m<2, T>(q, mode, p, st, prof);
+        case 4: return nest_rows_m<4, T>(q, mode, p, st, prof);
+        case 6: return nest_rows_m<6, T>(q, mode, p, st, prof);
     }
     return cudaErrorInvalidValue;
 }
 
 #define MOLT_NEST_ENTRY(T)                                                                                            \
+    template LineParams<T> nest_line_params<T>(const LineParams<T>&);                                                \
     template bool nest_rows_ok<T>(int);                                                                              \
     template bool nest_cols_ok<T>(int);                                                                              \
     template cudaError_t nest_cols<T>(const LineParams<T>&, int, const NestCols<T>&, cudaStream_t, long long*, Prof*); \

@@ -187,30 +187,232 @@ __device__ __forceinline__ void nest_finish(const NestCoef<typename N::V>& w, ty
     }
 }
 
-// The powers d^(cnt-1) of the two chunk lengths.
+// The same with the shifted wall stencils themselves (chunks of CNT > M nodes): the local integrals of the M/2 nodes
+// next to a wall are formed directly (wlA .. wrB) and the two-recurrence form starts behind them, where
+// no stencil leaves the line.
+template <class N, int M, int CNT, int KM>
+struct NestWall {
+    using V = typename N::V;
+    using T = typename N::T;
+    static constexpr int H = M / 2;
+    const LineParams<T>& lp;
+    const NestCoef<V>& w;
+    const V (&x)[KM];
+    __device__ __forceinline__ V sum(const T (&c)[kMaxStencil], int first) const {
+        V a = N::mul(N::splat(c[0]), x[first]);
+#pragma unroll
+        for (int o = 1; o <= M; ++o) a = N::fma(N::splat(c[o]), x[first + o], a);
+        return a;
+    }
+    // left wall: J^L_k (k = 1..H-1), J^R_k (k = 0..H-1); right wall: of node CNT-H+j
+    __device__ __forceinline__ V jla(int k) const { return sum(lp.wlA[k - 1], H); }
+    __device__ __forceinline__ V jra(int k) const { return sum(lp.wrA[k], H); }
+    __device__ __forceinline__ V jlb(int j) const { return sum(lp.wlB[j], H + CNT - 1 - M); }
+    __device__ __forceinline__ V jrb(int j) const { return sum(lp.wrB[j], H + CNT - 1 - M); }
+    // P^L_k - Q_k and P^R_k - R_k
+    __device__ __forceinline__ V bl(int k) const {
+        V a = N::mul(w.beta[1], x[k + 1]);
+#pragma unroll
+        for (int i = 2; i <= M; ++i) a = N::fma(w.beta[i], x[k + i], a);
+        return a;
+    }
+    __device__ __forceinline__ V br(int k) const {
+        V a = N::mul(w.beta[1], x[k + M - 1]);
+#pragma unroll
+        for (int i = 2; i <= M; ++i) a = N::fma(w.beta[i], x[k + M - i], a);
+        return a;
+    }
+};
+
+// As nest_agg, walls by their shifted stencils.
+template <class N, int M, int CNT, int KM>
+__device__ __forceinline__ void nest_agg_wall(const LineParams<typename N::T>& lp, const NestCoef<typename N::V>& w,
+                                         typename N::T pw, const NestChunk& c, const typename N::V (&x)[KM],
+                                         typename N::V& aL, typename N::V& aR) {
+    using V = typename N::V;
+    constexpr int H = M / 2;
+    const V dv = N::splat(lp.d), nd = N::splat(-lp.d), pv = N::splat(pw);
+    V s = x[0], r = x[CNT - 1 + M];
+#pragma unroll
+    for (int k = 1; k < CNT; ++k) {
+        s = N::fma(dv, s, x[k]);
+        r = N::fma(dv, r, x[CNT - 1 - k + M]);
+    }
+    V a = N::mul(w.alpha, s), b = N::mul(w.alpha, r);
+    V ka = N::mul(w.beta[1], x[0]), kb = N::mul(w.beta[1], x[CNT - 1 + M]);
+#pragma unroll
+    for (int i = 1; i <= M; ++i) {
+        a = N::fma(w.beta[i], x[CNT - 1 + i], a);
+        b = N::fma(w.beta[i], x[M - i], b);
+        if (i > 1) {
+            ka = N::fma(w.beta[i], x[i - 1], ka);
+            kb = N::fma(w.beta[i], x[CNT - i + M], kb);
+        }
+    }
+    aL = N::fma(pv, N::mul(nd, ka), a);
+    aR = N::fma(pv, N::mul(nd, kb), b);
+    if (c.mA | c.mB) {
+        const NestWall<N, M, CNT, KM> wl{lp, w, x};
+        const V m1 = N::splat(typename N::T(-1));
+        if (c.mA) {
+            V p = N::zero(), q = N::mul(nd, kb);   // kb: R just past the chunk is -kb
+#pragma unroll
+            for (int k = 1; k < H; ++k) p = N::fma(dv, p, wl.jla(k));
+            p = N::fma(m1, wl.bl(H - 1), p);
+#pragma unroll
+            for (int k = H; k < CNT; ++k) p = N::fma(dv, p, N::mul(w.alpha, x[k]));
+            q = N::add(q, N::mul(w.alpha, x[CNT - 1 + M]));
+#pragma unroll
+            for (int k = CNT - 2; k >= H; --k) q = N::fma(dv, q, N::mul(w.alpha, x[k + M]));
+            q = N::add(q, wl.br(H));
+#pragma unroll
+            for (int k = H - 1; k >= 0; --k) q = N::fma(dv, q, wl.jra(k));
+            aL = N::blend(aL, N::add(p, wl.bl(CNT - 1)), c.mA);
+            aR = N::blend(aR, q, c.mA);
+        }
+        if (c.mB) {
+            V p = N::mul(nd, ka), q = N::zero();   // Q just before the chunk is -ka
+#pragma unroll
+            for (int k = CNT - 2; k >= CNT - H; --k) q = N::fma(dv, q, wl.jrb(k - (CNT - H)));
+            q = N::fma(m1, wl.br(CNT - H), q);
+#pragma unroll
+            for (int k = CNT - H - 1; k >= 0; --k) q = N::fma(dv, q, N::mul(w.alpha, x[k + M]));
+            p = N::add(p, N::mul(w.alpha, x[0]));
+#pragma unroll
+            for (int k = 1; k < CNT - H; ++k) p = N::fma(dv, p, N::mul(w.alpha, x[k]));
+            p = N::add(p, wl.bl(CNT - 1 - H));
+#pragma unroll
+            for (int k = CNT - H; k < CNT; ++k) p = N::fma(dv, p, wl.jlb(k - (CNT - H)));
+            aL = N::blend(aL, p, c.mB);
+            aR = N::blend(aR, N::add(q, wl.br(0)), c.mB);
+        }
+    }
+}
+
+// As nest_finish, walls by their shifted stencils.
+template <class N, int K, int M, int CNT, int KM, class End>
+__device__ __forceinline__ void nest_finish_wall(const LineParams<typename N::T>& lp, const NestCoef<typename N::V>& w,
+                                            const NestChunk& c, const typename N::V (&x)[KM], typename N::V cL,
+                                            typename N::V cR, End end, typename N::V (&out)[K]) {
+    using V = typename N::V;
+    constexpr int H = M / 2;
+    const V dv = N::splat(lp.d), m1 = N::splat(typename N::T(-1));
+    const NestWall<N, M, CNT, KM> wl{lp, w, x};
+    V ka = N::mul(w.beta[1], x[0]), kb = N::mul(w.beta[1], x[CNT - 1 + M]);
+#pragma unroll
+    for (int i = 2; i <= M; ++i) {
+        ka = N::fma(w.beta[i], x[i - 1], ka);
+        kb = N::fma(w.beta[i], x[CNT - i + M], kb);
+    }
+    V q = N::fma(dv, N::fma(m1, ka, cL), N::mul(w.alpha, x[0]));
+    V r = N::fma(dv, N::fma(m1, kb, cR), N::mul(w.alpha, x[CNT - 1 + M]));
+    V pb[H];                      // right wall: P^R of the last H nodes
+#pragma unroll
+    for (int j = 0; j < H; ++j) pb[j] = N::zero();
+    V rs = N::zero();             // ... and R of node CNT - H
+    if (c.mB) {
+        pb[H - 1] = end(1);
+#pragma unroll
+        for (int j = H - 2; j >= 0; --j) pb[j] = N::fma(dv, pb[j + 1], wl.jrb(j));
+        rs = N::fma(m1, wl.br(CNT - H), pb[0]);
+    }
+    out[CNT - 1] = r;
+#pragma unroll
+    for (int k = CNT - 2; k >= 0; --k) {
+        r = N::fma(dv, r, N::mul(w.alpha, x[k + M]));
+        if (k == CNT - H && H > 1 && c.mB) r = N::blend(r, rs, c.mB);
+        out[k] = r;
+        if (k == CNT - 1 - H && H == 1 && c.mB) {   // H = 1: the start is the last node itself
+            r = N::blend(r, N::fma(dv, rs, N::mul(w.alpha, x[k + M])), c.mB);
+            out[k] = r;
+        }
+    }
+    V pa[H], qs = N::zero();      // left wall: the first H outputs, Q of node H - 1
+#pragma unroll
+    for (int j = 0; j < H; ++j) pa[j] = N::zero();
+    if (c.mA) {
+        V p = N::add(out[H], wl.br(H));
+#pragma unroll
+        for (int k = H - 1; k >= 0; --k) {
+            p = N::fma(dv, p, wl.jra(k));
+            pa[k] = p;
+        }
+        p = end(0);
+        pa[0] = N::add(pa[0], p);
+#pragma unroll
+        for (int k = 1; k < H; ++k) {
+            p = N::fma(dv, p, wl.jla(k));
+            pa[k] = N::add(pa[k], p);
+        }
+        qs = N::fma(m1, wl.bl(H - 1), p);
+    }
+    V ql = N::zero();             // Q of node CNT - 1 - H
+#pragma unroll
+    for (int k = 0; k < CNT; ++k) {
+        if (k > 0) q = N::fma(dv, q, N::mul(w.alpha, x[k]));
+        if (k == H - 1 && c.mA) q = N::blend(q, qs, c.mA);
+        if (k == CNT - 1 - H) ql = q;
+        V e = N::fma(w.gamma[H], x[k + H], N::add(out[k], q));
+#pragma unroll
+        for (int m = 0; m < H; ++m) e = N::fma(w.gamma[m], N::add(x[k + m], x[k + M - m]), e);
+        out[k] = e;
+    }
+    if (c.mA) {
+#pragma unroll
+        for (int k = 0; k < H; ++k) out[k] = N::blend(out[k], pa[k], c.mA);
+    }
+    if (c.mB) {
+        V p = N::add(ql, wl.bl(CNT - 1 - H));
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            p = N::fma(dv, p, wl.jlb(j));
+            out[CNT - H + j] = N::blend(out[CNT - H + j], N::add(pb[j], p), c.mB);
+        }
+    }
+}
+
+// Walls by ghost values or by shifted stencils.  Sixth order's ghosts weigh the first nodes by up to 140, which on rough data
+// costs FP32 two bits of the nodes beside a wall (1024^2 Neumann, two solves: largest error 3.5e-6 of the field's largest value
+// with ghosts, 7.4e-7 with the stencils, 8.0e-7 by single sweeps); fourth order's (up to 10) cost nothing
+// measurable (8.2e-7, 8.7e-7, 7.0e-7), and in FP64 neither does (256^2 to 1024^2: 1.3e-14 and 1.8e-14 of either form and of
+// single sweeps).  The stencils are work for the warps that hold a wall, which are all of them on short FP64 lines:
+// 256^2 FP64 117 us an iteration, with ghosts 80.
+template <class N, int M> inline constexpr bool kNestGhosts = M <= 4 || sizeof(typename N::T) == 8;
+
+// The powers d^(K-1) and d^(K-2): what a value decays by over a chunk of K or K - 1 nodes, one node less.
 template <typename T> struct NestPow { T full, less; };
 
 template <class N, int K, int M, int S, bool RAG, int KM>
-__device__ __forceinline__ void nest_chunk_agg(const NestCoef<typename N::V>& w, typename N::T d,
+__device__ __forceinline__ void nest_chunk_agg(const LineParams<typename N::T>& lp, const NestCoef<typename N::V>& w,
                                                const NestPow<typename N::T>& p, const NestChunk& c,
                                                typename N::V (&x)[KM], typename N::V& aL, typename N::V& aR) {
-    if (!RAG || c.cnt == K) {
-        nest_ghosts<N, M, K>(c, x);
-        nest_agg<N, M, K>(w, d, p.full, c, x, aL, aR);
+    if constexpr (kNestGhosts<N, M>) {
+        if (!RAG || c.cnt == K) {
+            nest_ghosts<N, M, K>(c, x);
+            nest_agg<N, M, K>(w, lp.d, p.full, c, x, aL, aR);
+        } else {
+            nest_ghosts<N, M, K - S>(c, x);
+            nest_agg<N, M, K - S>(w, lp.d, p.less, c, x, aL, aR);
+        }
     } else {
-        nest_ghosts<N, M, K - S>(c, x);
-        nest_agg<N, M, K - S>(w, d, p.less, c, x, aL, aR);
+        if (!RAG || c.cnt == K) nest_agg_wall<N, M, K>(lp, w, p.full, c, x, aL, aR);
+        else nest_agg_wall<N, M, K - S>(lp, w, p.less, c, x, aL, aR);
     }
     if (c.cnt == 0) aL = aR = N::zero();
 }
 
 // end(0), end(1): the boundary values of the line, asked for at walls only.
 template <class N, int K, int M, int S, bool RAG, int KM, class End>
-__device__ __forceinline__ void nest_chunk_finish(const NestCoef<typename N::V>& w, typename N::T d, const NestChunk& c,
-                                                  const typename N::V (&x)[KM], typename N::V cL, typename N::V cR,
-                                                  End end, typename N::V (&out)[K]) {
-    if (!RAG || c.cnt == K) nest_finish<N, K, M, K>(w, d, c, x, cL, cR, end, out);
-    else nest_finish<N, K, M, K - S>(w, d, c, x, cL, cR, end, out);
+__device__ __forceinline__ void nest_chunk_finish(const LineParams<typename N::T>& lp, const NestCoef<typename N::V>& w,
+                                                  const NestChunk& c, const typename N::V (&x)[KM], typename N::V cL,
+                                                  typename N::V cR, End end, typename N::V (&out)[K]) {
+    if constexpr (kNestGhosts<N, M>) {
+        if (!RAG || c.cnt == K) nest_finish<N, K, M, K>(w, lp.d, c, x, cL, cR, end, out);
+        else nest_finish<N, K, M, K - S>(w, lp.d, c, x, cL, cR, end, out);
+    } else {
+        if (!RAG || c.cnt == K) nest_finish_wall<N, K, M, K>(lp, w, c, x, cL, cR, end, out);
+        else nest_finish_wall<N, K, M, K - S>(lp, w, c, x, cL, cR, end, out);
+    }
 }
 
 // Halo values hl (before the chunk) and hr (after it) into the window x.
@@ -281,10 +483,12 @@ __device__ __forceinline__ unsigned long long nest_from_bits(unsigned long long 
 //     the y part of the iteration whose x part is w + E + H (B + H A) (solver.cpp);
 //   3D z pass:  outputs a3 = t, b3 = -2s + 4t - beta a, c3 = -w + 4s - 4t + beta (3a - b);
 //   copy: out = H H in.
-// Bound: issue slots and the latency of the scan's barriers (1.5 of 4 instructions a cycle, 24 warps a SM), not
-// memory: 4096^2 Neumann FP32 192 us = 1750 GB/s of its 20 B a point, the row pass 74 us.  K = 8 keeps the kernel
-// at 80 registers, three blocks a SM; K = 16 (two blocks) took 178 us there but 121 KB a block with the
-// arrays below, one block a SM, and 32-byte row segments (4 values) let one block hold 512 nodes.
+// Bound: issue slots and the latency of the scan's barriers (1.5 to 1.9 of 4 instructions a cycle, 16 warps a SM), not
+// memory: 4096^2 Neumann FP32 198 us = 1700 GB/s of its 20 B a point, the row pass 80 us.  Two blocks a SM with 128
+// registers, chunks of K = 8: 4096^2 Neumann FP32 276 us an iteration, vector model 593, 2048^2 78, 1001 x 777 37;
+// three blocks at 80 registers spill and take 300, 674, 87 and 40 (M = 6, 4096^2: 298 against 337).  The copy of up
+// to fourth order fits 80 registers: its three blocks give 250 us for the right side against 267.  K = 16 needs
+// 121 KB a block for the arrays below, one block a SM.  32-byte row segments (4 values) let one block hold 512 nodes.
 template <typename T>
 struct NestColArgs {
     const T* in0;
@@ -559,7 +763,7 @@ __device__ __forceinline__ typename N::V nest_vch(typename N::V x1, typename N::
 __device__ __forceinline__ void nest_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // Window of a field's column chunk from global memory: rows wrapped on periodic columns, clamped at walls
-// (the ghosts replace those values).
+// (ghosts replace those values, or no stencil uses them).
 template <class N, int K, int M, bool RAG, bool WIDE, int KM>
 __device__ __forceinline__ void nest_col_window(const typename N::T* f, const NestColGeo& g, int n, bool periodic, int ld,
                                                 typename N::V (&x)[KM]) {
@@ -587,10 +791,11 @@ __host__ __device__ constexpr int nest_col_pitch() {
     return NA == 1 ? K + 1 : NA * K + M + 1;
 }
 
+
 // FORM 0: every chunk of every block has K nodes and the blocks' chunks come in multiples of 16; 1: chunks
 // of K nodes; 2: chunks of K and K - 1 nodes.
 template <class N, int M, int FORM, bool WIDE, int MODE>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, MODE == NEST_COPY && M <= 4 ? 3 : 2)
 nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
                  const __grid_constant__ NestCoef<typename N::V> w,
                  const __grid_constant__ NestColArgs<typename N::T> a) {
@@ -610,8 +815,6 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     V* own = reinterpret_cast<V*>(nest_sm) + threadIdx.x * PITCH;
     auto arr = [&](int f, int k) -> V& { return own[f * K + k]; };
     auto end1 = [&](int h) -> V& { return own[NA * K + h]; };
-    const T d = lp.d;
-
     V x[K + M], hl[H], hr[H];   // hl, hr: the window's ends of field 0
     // ---- windows of the fields: nodes to shared memory, ends to hl / hr ----
     auto keep = [&](int q) {
@@ -722,13 +925,13 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
         for (int q = 0; q < NF; ++q) {
             window(q);
             V aL, aR;
-            nest_chunk_agg<N, K, M, S, RAG>(w, d, a.pw, ck, x, aL, aR);
+            nest_chunk_agg<N, K, M, S, RAG>(lp, w, a.pw, ck, x, aL, aR);
             if (g.slot < a.slots) {
                 V* e = ex + 2 * ((q << a.lcp) + g.cpi) * (a.slots + 4) + g.slot;
                 e[0] = aL;
                 e[a.slots + 4] = aR;
             }
-            if (ck.mA | ck.mB) {   // the ghosts
+            if (kNestGhosts<N, M> && (ck.mA | ck.mB)) {   // the ghosts
                 keep_ends(q);
                 if (RAG) arr(q, K - 1) = x[H + K - 1];
             }
@@ -760,7 +963,7 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
             }
         };
         auto finish = [&](int q) {
-            nest_chunk_finish<N, K, M, S, RAG>(w, d, ck, x, nest_col_carry<N, NF>(lp, c, sh, q, 0),
+            nest_chunk_finish<N, K, M, S, RAG>(lp, w, ck, x, nest_col_carry<N, NF>(lp, c, sh, q, 0),
                                                nest_col_carry<N, NF>(lp, c, sh, q, 1),
                                                [&](int dir) { return nest_col_end<N, NF>(lp, c, sh, q, dir); }, out);
         };

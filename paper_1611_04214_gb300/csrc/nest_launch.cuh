@@ -25,15 +25,13 @@ inline void nest_put(unsigned long long* o, double v) {
 template <typename T>
 void nest_put(T* o, double v) { *o = static_cast<T>(v); }
 
-// Coefficients of an inverse (NestCoef).  The quadrature weights are those of nu' = -ln d for the
-// decay d as the kernel holds it: the recurrence and the weights then belong to one operator (H 1 = 1
-// holds with a rounded d too).
+// Coefficients of an inverse (NestCoef) of nest_line_params, the quadrature weights in FP64.
 template <typename V, int M, typename T>
 NestCoef<V> nest_coef(const LineParams<T>& lp) {
     NestCoef<V> c;
     std::memset(&c, 0, sizeof(c));
     const double d = static_cast<double>(lp.d);
-    const double nu = d > 0.0 && d < 1.0 ? -std::log(d) : static_cast<double>(lp.nu);
+    const double nu = sizeof(T) == 4 && d > 0.0 && d < 1.0 ? -std::log(d) : static_cast<double>(lp.nu);
     int offs[M + 1];
     double w[M + 1], beta[M + 1];
     for (int o = 0; o <= M; ++o) offs[o] = o - M / 2;
@@ -52,7 +50,8 @@ NestPow<T> nest_pow(const LineParams<T>& lp, int K) {
     return {static_cast<T>(std::pow(d, K - 1)), static_cast<T>(std::pow(d, K - 2))};
 }
 
-template <typename T, int M, int FORM, bool WIDE, int MODE>
+// One column kernel, F::kern(); F::kPitch values per thread, F::kNF fields.
+template <class F, int M, typename T>
 cudaError_t nest_cols_run(const LineParams<T>& lp, const NestCols<T>& p, cudaStream_t st, Prof* prof) {
     using N = NestVec<T, sizeof(T) == 4 ? 2 : 1>;
     NestColArgs<T> a{};
@@ -66,10 +65,9 @@ cudaError_t nest_cols_run(const LineParams<T>& lp, const NestCols<T>& p, cudaStr
     a.pw = nest_pow(lp, kNestColK);
     a.exact = static_cast<double>(lp.nu) * lp.N < 45.0;   // e^-45 < 2^-64
     const int nt = ((a.slots << a.lcp) + 31) / 32 * 32;
-    constexpr int NA = MODE == NEST_COPY ? 1 : 3, NF = MODE == NEST_COPY ? 1 : 2;
-    const size_t smem = static_cast<size_t>(nt) * (nest_col_pitch<kNestColK, M, NA>() * sizeof(typename N::V) + 4 * sizeof(T)) +
-                        (static_cast<size_t>(2 * NF * (a.slots + 4)) << a.lcp) * sizeof(typename N::V);
-    auto kern = nest_cols_kernel<N, M, FORM, WIDE, MODE>;
+    const size_t smem = static_cast<size_t>(nt) * (F::kPitch * sizeof(typename N::V) + 4 * sizeof(T)) +
+                        (static_cast<size_t>(2 * F::kNF * (a.slots + 4)) << a.lcp) * sizeof(typename N::V);
+    auto kern = F::kern();
     static int limit = [&] {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return -1;
         return smem_optin(kern);
@@ -88,64 +86,70 @@ cudaError_t nest_cols_run(const LineParams<T>& lp, const NestCols<T>& p, cudaStr
     cfg.attrs = attr;
     cfg.numAttrs = a.C > 1 ? 1 : 0;
     const NestCoef<typename N::V> w = nest_coef<typename N::V, M>(lp);
-    prof_begin(prof, MODE == NEST_COPY ? kProfNestColsRhs : kProfNestCols, st);
+    prof_begin(prof, F::kSlot, st);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, lp, w, a);
     prof_end(prof, st);
     return e;
 }
 
-template <class N, int M, bool RAG, bool WARP, int MODE>
-cudaError_t nest_rows_launch(const LineParams<typename N::T>& lp, const NestRowArgs<typename N::T>& a_in, cudaStream_t st,
-                             Prof* prof) {
-    auto kern = nest_rows_kernel<N, M, RAG, WARP, MODE>;
-    const int block = WARP ? 128 : a_in.TL;
-    const int per = WARP ? block / a_in.TL : 1;
-    const size_t smem = WARP ? 0 : static_cast<size_t>(2 * M) * a_in.TL * sizeof(typename N::V);
-    static int limit = smem_optin(kern);
+template <typename T, int M, int FORM, bool WIDE, int MODE> struct NestColsPass {
+    static constexpr int kPitch = nest_col_pitch<kNestColK, M, MODE == NEST_COPY ? 1 : 3>();
+    static constexpr int kNF = MODE == NEST_COPY ? 1 : 2, kSlot = MODE == NEST_COPY ? kProfNestColsRhs : kProfNestCols;
+    static auto kern() { return nest_cols_kernel<NestVec<T, sizeof(T) == 4 ? 2 : 1>, M, FORM, WIDE, MODE>; }
+};
+
+// One row kernel, F::kern(); args has the layout but for `ahead`.
+template <class F, class N, int M, bool WARP, class Args>
+cudaError_t nest_rows_launch(const LineParams<typename N::T>& lp, Args a, cudaStream_t st, Prof* prof, int slot) {
+    const int block = WARP ? 128 : a.TL;
+    const int per = WARP ? block / a.TL : 1;
+    const size_t smem = WARP ? 0 : static_cast<size_t>(2 * M) * a.TL * sizeof(typename N::V);
+    static int limit = smem_optin(F::kern());
     if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
     const NestCoef<typename N::V> w = nest_coef<typename N::V, M>(lp);
-    NestRowArgs<typename N::T> a = a_in;
-    // two blocks a SM (the kernel's launch bounds); lines that stay in L2 anyway need no fetching ahead
+    // two blocks a SM (the kernel's launch bounds); short lines are on their way before they are wanted
     a.ahead = WARP ? 0 : 2 * 152;
-    prof_begin(prof, MODE == NEST_ROW_COPY ? kProfNestRowsRhs : kProfNestRows, st);
-    kern<<<(a.nlines + per - 1) / per, block, smem, st>>>(lp, w, a);
+    prof_begin(prof, slot, st);
+    F::kern()<<<(a.nlines + per - 1) / per, block, smem, st>>>(lp, w, a);
     prof_end(prof, st);
     return cudaGetLastError();
 }
 
-template <class N, int M, int MODE>
-cudaError_t nest_rows_team(const LineParams<typename N::T>& lp, NestRowArgs<typename N::T>& a, bool rag, cudaStream_t st,
-                           Prof* prof) {
+// Lines cut into chunks of one length or two (RAG), teams within a warp or of a block.  F<N, M, RAG, WARP>::kern()
+// is the kernel.
+template <class N, int M, template <class, int, bool, bool> class F, class Args>
+cudaError_t nest_rows_team(const LineParams<typename N::T>& lp, Args a, cudaStream_t st, Prof* prof, int slot) {
     const int nc = a.cut.nc;
-    if (nc <= 32) {
-        a.TL = 1;
-        while (a.TL < nc) a.TL *= 2;
-        if constexpr (N::W == 1)
-            if (rag) return nest_rows_launch<N, M, true, true, MODE>(lp, a, st, prof);
-        return nest_rows_launch<N, M, false, true, MODE>(lp, a, st, prof);
-    }
+    const bool warp = nc <= 32, rag = N::W == 1 && a.cut.rem != nc;
     a.TL = (nc + 31) / 32 * 32;
-    if constexpr (N::W == 1)
-        if (rag) return nest_rows_launch<N, M, true, false, MODE>(lp, a, st, prof);
-    return nest_rows_launch<N, M, false, false, MODE>(lp, a, st, prof);
+    if (warp)
+        for (a.TL = 1; a.TL < nc;) a.TL *= 2;
+    if constexpr (N::W == 1) {
+        if (rag)
+            return warp ? nest_rows_launch<F<N, M, true, true>, N, M, true>(lp, a, st, prof, slot)
+                        : nest_rows_launch<F<N, M, true, false>, N, M, false>(lp, a, st, prof, slot);
+    }
+    return warp ? nest_rows_launch<F<N, M, false, true>, N, M, true>(lp, a, st, prof, slot)
+                : nest_rows_launch<F<N, M, false, false>, N, M, false>(lp, a, st, prof, slot);
 }
+template <class N, int M, bool RAG, bool WARP> struct NestRowPass {
+    static auto kern() { return nest_rows_kernel<N, M, RAG, WARP, NEST_ROW_PASS>; }
+};
+template <class N, int M, bool RAG, bool WARP> struct NestRowCopy {
+    static auto kern() { return nest_rows_kernel<N, M, RAG, WARP, NEST_ROW_COPY>; }
+};
 
-template <typename T, int M, int MODE>
-cudaError_t nest_rows_run(const LineParams<T>& lp, const NestRows<T>& p, cudaStream_t st, Prof* prof) {
-    NestRowArgs<T> a{};
-    a.A = p.A, a.B = p.B, a.E = p.E, a.w = p.w, a.nlines = p.nlines, a.fix = p.fix, a.wall = p.wall, a.red = p.red;
+template <typename T, int M, template <class, int, bool, bool> class F, class Args>
+cudaError_t nest_rows_run(const LineParams<T>& lp, Args a, int nlines, bool aligned, cudaStream_t st, Prof* prof, int slot) {
     int W;
-    if (!nest_row_shape<T>(lp.n, &W, &a.cut)) return cudaErrorInvalidValue;
-    const T* fields[] = {p.A, p.B, p.E, p.w};
-    for (const T* f : fields)
-        if (W == 2 && !aligned16(f)) return cudaErrorInvalidValue;
+    if (!nest_row_shape<T>(lp.n, &W, &a.cut) || (W == 2 && !aligned)) return cudaErrorInvalidValue;
+    a.nlines = nlines;
     a.half = lp.n / W;
     a.pw = nest_pow(lp, kNestRowK);
-    const bool rag = a.cut.rem != a.cut.nc;
     if constexpr (sizeof(T) == 4) {
-        if (W == 2) return nest_rows_team<NestVec<float, 2>, M, MODE>(lp, a, rag, st, prof);
+        if (W == 2) return nest_rows_team<NestVec<float, 2>, M, F>(lp, a, st, prof, slot);
     }
-    return nest_rows_team<NestVec<T, 1>, M, MODE>(lp, a, rag, st, prof);
+    return nest_rows_team<NestVec<T, 1>, M, F>(lp, a, st, prof, slot);
 }
 
 }  // namespace detail
@@ -162,12 +166,12 @@ cudaError_t nest_cols_mode(const LineParams<T>& lp, const NestCols<T>& p, cudaSt
     const int form = lp.n % kNestColK != 0 ? 2 : nc % (16 * C) != 0 ? 1 : 0;
     if constexpr (sizeof(T) == 4) {
         if (!wide)
-            return form == 2 ? nest_cols_run<T, M, 2, false, MODE>(lp, p, st, prof)
-                             : nest_cols_run<T, M, 1, false, MODE>(lp, p, st, prof);
+            return form == 2 ? nest_cols_run<NestColsPass<T, M, 2, false, MODE>, M>(lp, p, st, prof)
+                             : nest_cols_run<NestColsPass<T, M, 1, false, MODE>, M>(lp, p, st, prof);
     }
-    return form == 2   ? nest_cols_run<T, M, 2, true, MODE>(lp, p, st, prof)
-           : form == 1 ? nest_cols_run<T, M, 1, true, MODE>(lp, p, st, prof)
-                       : nest_cols_run<T, M, 0, true, MODE>(lp, p, st, prof);
+    return form == 2   ? nest_cols_run<NestColsPass<T, M, 2, true, MODE>, M>(lp, p, st, prof)
+           : form == 1 ? nest_cols_run<NestColsPass<T, M, 1, true, MODE>, M>(lp, p, st, prof)
+                       : nest_cols_run<NestColsPass<T, M, 0, true, MODE>, M>(lp, p, st, prof);
 }
 }  // namespace detail
 
@@ -185,8 +189,11 @@ cudaError_t nest_cols_m(const LineParams<T>& lp, int mode, const NestCols<T>& p,
 template <int M, typename T>
 cudaError_t nest_rows_m(const LineParams<T>& lp, int mode, const NestRows<T>& p, cudaStream_t st, Prof* prof) {
     using namespace detail;
-    return mode == NEST_ROW_PASS ? nest_rows_run<T, M, NEST_ROW_PASS>(lp, p, st, prof)
-                                 : nest_rows_run<T, M, NEST_ROW_COPY>(lp, p, st, prof);
+    NestRowArgs<T> a{};
+    a.A = p.A, a.B = p.B, a.E = p.E, a.w = p.w, a.fix = p.fix, a.wall = p.wall, a.red = p.red;
+    const bool al = aligned16(p.A) && aligned16(p.B) && aligned16(p.E) && aligned16(p.w);
+    return mode == NEST_ROW_PASS ? nest_rows_run<T, M, NestRowPass>(lp, a, p.nlines, al, st, prof, kProfNestRows)
+                                 : nest_rows_run<T, M, NestRowCopy>(lp, a, p.nlines, al, st, prof, kProfNestRowsRhs);
 }
 
 #define MOLT_INSTANTIATE_NEST(M, T)                                                                                  \

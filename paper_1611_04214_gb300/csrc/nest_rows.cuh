@@ -13,21 +13,26 @@
 
 namespace molt {
 
+// How the lines are laid over threads.
 template <typename T>
-struct NestRowArgs {
-    const T* A;
-    const T* B;
-    const T* E;
-    T* w;            // pass: the iterate, in place; copy: the output
+struct NestRowLayout {
     int nlines;
     int half;        // nodes of a register half (n or n / 2)
     int TL;          // threads per line
     NestCut cut;     // of a half
+    NestPow<T> pw;   // d^(cnt-1) of the two chunk lengths
+    int ahead;       // lines resident at a time (0: nothing is fetched ahead)
+};
+
+template <typename T>
+struct NestRowArgs : NestRowLayout<T> {
+    const T* A;
+    const T* B;
+    const T* E;
+    T* w;            // pass: the iterate, in place; copy: the output
     int fix;         // Dirichlet grids: write `wall` to the wall nodes
     T wall;
     unsigned long long* red;
-    NestPow<T> pw;   // d^(cnt-1) of the two chunk lengths
-    int ahead;       // lines resident at a time (0: nothing is fetched ahead)
 };
 
 template <class N>
@@ -239,6 +244,135 @@ __device__ __forceinline__ void nest_reduce(RedAcc<T> r, unsigned long long* slo
     }
 }
 
+// A thread's place: its line, chunk and the constants of the scans.
+template <class N>
+struct NestRowThread {
+    using T = typename N::T;
+    NestRowScan<T> c;
+    NestChunk ck;
+    int line, start;
+    bool on;          // the thread has nodes of a line
+    size_t row;       // offset of the line
+};
+
+template <class N, int K, bool RAG, bool WARP>
+__device__ __forceinline__ NestRowThread<N> nest_row_thread(const LineParams<typename N::T>& lp,
+                                                            const NestRowLayout<typename N::T>& a) {
+    using T = typename N::T;
+    constexpr int S = 1;
+    NestRowThread<N> g;
+    NestRowScan<T>& c = g.c;
+    c.lane = threadIdx.x & 31;
+    c.warp = threadIdx.x >> 5;
+    c.nwarps = blockDim.x >> 5;
+    c.width = a.TL < 32 ? a.TL : 32;
+    if constexpr (WARP) {
+        c.tl = c.lane & (a.TL - 1);
+        g.line = (blockIdx.x * c.nwarps + c.warp) * (32 / a.TL) + c.lane / a.TL;
+    } else {
+        c.tl = threadIdx.x;
+        g.line = blockIdx.x;
+    }
+    const bool live = c.tl < a.cut.nc;
+    g.on = live && g.line < a.nlines;
+    const int ci = live ? c.tl : 0;
+    g.ck.cnt = !live ? 0 : (!RAG || ci < a.cut.rem) ? K : K - S;
+    g.start = RAG ? ci * (K - S) + S * min(ci, a.cut.rem) : ci * K;
+    const bool periodic = lp.bc == BC_PERIODIC;
+    g.ck.mA = live && !periodic && ci == 0 ? 1 : 0;
+    g.ck.mB = live && !periodic && ci == a.cut.nc - 1 ? N::W : 0;
+    g.row = static_cast<size_t>(g.on ? g.line : 0) * lp.n;
+    return g;
+}
+
+// The scans' constants of a thread (after the first loads have been issued).
+template <class N, int K, bool RAG, bool WARP>
+__device__ __forceinline__ void nest_row_scan_setup(const LineParams<typename N::T>& lp,
+                                                    const NestRowLayout<typename N::T>& a, NestRowThread<N>& g,
+                                                    NestRowShared<N>& sh) {
+    using T = typename N::T;
+    NestRowScan<T>& c = g.c;
+    const int cnt = g.ck.cnt;
+    const T D = cnt == 0 ? T(1) : (!RAG || cnt == K) ? a.pw.full * lp.d : a.pw.less * lp.d;
+    T f = D, b = D;
+    const int li = c.lane & (c.width - 1);
+#pragma unroll
+    for (int s = 0; s < 5; ++s) {
+        const int o = 1 << s;
+        c.df[s] = f;
+        c.db[s] = b;
+        if (o < c.width) {
+            const T u = __shfl_up_sync(kFull, f, o, c.width), v = __shfl_down_sync(kFull, b, o, c.width);
+            if (li >= o) f *= u;
+            if (li + o < c.width) b *= v;
+        }
+    }
+    c.Dxf = __shfl_up_sync(kFull, f, 1, c.width);
+    c.Dxb = __shfl_down_sync(kFull, b, 1, c.width);
+    if (li == 0) c.Dxf = T(1);
+    if (li == c.width - 1) c.Dxb = T(1);
+    c.Dh = dev_exp(-lp.nu * T(a.half));
+    const int last = g.start + cnt;
+#pragma unroll
+    for (int q = 0; q < N::W; ++q) {
+        const int p = q * a.half, m = lp.bc == BC_PERIODIC ? 0 : 1;   // a wall's value starts one node later
+        c.pl[q] = dev_exp(-lp.nu * T(max(p + g.start - m, 0)));
+        c.pr[q] = dev_exp(-lp.nu * T(max(lp.n - p - last - m, 0)));
+    }
+    if constexpr (N::W == 1) c.pl[1] = c.pr[1] = T(0);
+    if constexpr (!WARP) {
+        if (c.lane == 31) sh.wd[c.warp] = f;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            T p = T(1);
+            for (int w = 0; w < c.nwarps; ++w) {
+                sh.wdf[w] = p;
+                p *= sh.wd[w];
+            }
+            p = T(1);
+            for (int w = c.nwarps - 1; w >= 0; --w) {
+                sh.wdb[w] = p;
+                p *= sh.wd[w];
+            }
+        }
+    }
+}
+
+// x (the window's own nodes set) <- H x: the outputs in out, the window's ends completed.
+template <class N, int K, int M, bool RAG, bool WARP, int KM>
+__device__ __forceinline__ void nest_row_inverse(const LineParams<typename N::T>& lp,
+                                                 const NestCoef<typename N::V>& w,
+                                                 const NestRowLayout<typename N::T>& a, const NestRowThread<N>& g,
+                                                 NestRowShared<N>& sh, typename N::V* edge, typename N::V (&x)[KM],
+                                                 typename N::V (&out)[K]) {
+    using V = typename N::V;
+    V aL, aR, cL, cR, XL, XR;
+    nest_row_halo<N, K, M, 1, RAG, WARP>(g.c, a.cut.nc, g.ck.cnt, edge, a.TL, x);
+    nest_chunk_agg<N, K, M, 1, RAG>(lp, w, a.pw, g.ck, x, aL, aR);
+    nest_row_scan<N, WARP>(lp, g.c, sh, aL, aR, cL, cR, XL, XR);
+    nest_chunk_finish<N, K, M, 1, RAG>(lp, w, g.ck, x, cL, cR, [&](int dir) { return dir ? XR : XL; }, out);
+}
+
+// value(k), the thread's k-th node, to a field.
+template <class N, int K, bool RAG, class F>
+__device__ __forceinline__ void nest_row_store(typename N::T* f, int half, int start, int cnt, F value) {
+    using T = typename N::T;
+    if constexpr (N::W == 2) {
+#pragma unroll
+        for (int j = 0; j < K / 4; ++j) {
+            const typename N::V a = value(4 * j), b = value(4 * j + 1), c = value(4 * j + 2), d = value(4 * j + 3);
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                *reinterpret_cast<float4*>(f + q * half + start + 4 * j) =
+                    make_float4(N::get(a, q), N::get(b, q), N::get(c, q), N::get(d, q));
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (!RAG || k < cnt) f[start + k] = value(k);
+    }
+}
+
 template <class N, int M, bool RAG, bool WARP, int MODE>
 __global__ void __launch_bounds__(N::W == 2 ? 256 : 512, N::W == 2 ? 2 : 1)
 nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
@@ -246,40 +380,21 @@ nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
                  const __grid_constant__ NestRowArgs<typename N::T> a) {
     using V = typename N::V;
     using T = typename N::T;
-    constexpr int K = kNestRowK, H = M / 2, S = 1;
+    constexpr int K = kNestRowK, H = M / 2;
     extern __shared__ __align__(16) unsigned char nest_row_sm[];
     V* edge = reinterpret_cast<V*>(nest_row_sm);      // two sets of 2 H values per thread (block teams)
     __shared__ NestRowShared<N> sh;
-    NestRowScan<T> c;
-    c.lane = threadIdx.x & 31;
-    c.warp = threadIdx.x >> 5;
-    c.nwarps = blockDim.x >> 5;
-    c.width = a.TL < 32 ? a.TL : 32;
-    int line;
-    if constexpr (WARP) {
-        c.tl = c.lane & (a.TL - 1);
-        line = (blockIdx.x * c.nwarps + c.warp) * (32 / a.TL) + c.lane / a.TL;
-    } else {
-        c.tl = threadIdx.x;
-        line = blockIdx.x;
-    }
-    const bool live = c.tl < a.cut.nc, on = live && line < a.nlines;
-    const int ci = live ? c.tl : 0;
-    NestChunk ck;
-    ck.cnt = !live ? 0 : (!RAG || ci < a.cut.rem) ? K : K - S;
-    const int start = RAG ? ci * (K - S) + S * min(ci, a.cut.rem) : ci * K;
-    const bool periodic = lp.bc == BC_PERIODIC;
-    ck.mA = live && !periodic && ci == 0 ? 1 : 0;
-    ck.mB = live && !periodic && ci == a.cut.nc - 1 ? N::W : 0;
-    const size_t row = static_cast<size_t>(on ? line : 0) * lp.n;
+    NestRowThread<N> g = nest_row_thread<N, K, RAG, WARP>(lp, a);
+    const int start = g.start, cnt = g.ck.cnt, line = g.line;
+    const size_t row = g.row;
 
-    V x[K + M];
-    nest_row_load<N, K, RAG, H>(a.A + row, a.half, start, ck.cnt, on, x);
+    V x[K + M], out[K];
+    nest_row_load<N, K, RAG, H>(a.A + row, a.half, start, cnt, g.on, x);
     if (a.ahead) {
         // the fields that this line needs later, and the first one of the line after the resident ones, into L2
         const int step = 128 / sizeof(T);
         const size_t next = static_cast<size_t>(line + a.ahead < a.nlines ? line + a.ahead : a.nlines - 1) * lp.n;
-        for (int p = c.tl * step; p < lp.n; p += a.TL * step) {
+        for (int p = g.c.tl * step; p < lp.n; p += a.TL * step) {
             if constexpr (MODE == NEST_ROW_PASS) {
                 nest_prefetch(a.B + row + p);
                 nest_prefetch(a.E + row + p);
@@ -288,86 +403,19 @@ nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
             nest_prefetch(a.A + next + p);
         }
     }
+    nest_row_scan_setup<N, K, RAG, WARP>(lp, a, g, sh);
 
-    // ---- scan constants ----
-    {
-        const T D = ck.cnt == 0 ? T(1) : (!RAG || ck.cnt == K) ? a.pw.full * lp.d : a.pw.less * lp.d;
-        T f = D, b = D;
-        const int li = c.lane & (c.width - 1);
-#pragma unroll
-        for (int s = 0; s < 5; ++s) {
-            const int o = 1 << s;
-            c.df[s] = f;
-            c.db[s] = b;
-            if (o < c.width) {
-                const T u = __shfl_up_sync(kFull, f, o, c.width), v = __shfl_down_sync(kFull, b, o, c.width);
-                if (li >= o) f *= u;
-                if (li + o < c.width) b *= v;
-            }
-        }
-        c.Dxf = __shfl_up_sync(kFull, f, 1, c.width);
-        c.Dxb = __shfl_down_sync(kFull, b, 1, c.width);
-        if (li == 0) c.Dxf = T(1);
-        if (li == c.width - 1) c.Dxb = T(1);
-        c.Dh = dev_exp(-lp.nu * T(a.half));
-        const int last = start + ck.cnt;
-#pragma unroll
-        for (int q = 0; q < N::W; ++q) {
-            const int p = q * a.half, m = periodic ? 0 : 1;   // a wall's value starts one node later
-            c.pl[q] = dev_exp(-lp.nu * T(max(p + start - m, 0)));
-            c.pr[q] = dev_exp(-lp.nu * T(max(lp.n - p - last - m, 0)));
-        }
-        if constexpr (N::W == 1) c.pl[1] = c.pr[1] = T(0);
-        if constexpr (!WARP) {
-            if (c.lane == 31) sh.wd[c.warp] = f;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                T p = T(1);
-                for (int w = 0; w < c.nwarps; ++w) {
-                    sh.wdf[w] = p;
-                    p *= sh.wd[w];
-                }
-                p = T(1);
-                for (int w = c.nwarps - 1; w >= 0; --w) {
-                    sh.wdb[w] = p;
-                    p *= sh.wd[w];
-                }
-            }
-        }
-    }
-    const T d = lp.d;
-    V aL, aR, cL, cR, XL, XR, out[K];
-    nest_row_halo<N, K, M, S, RAG, WARP>(c, a.cut.nc, ck.cnt, edge, a.TL, x);
-    nest_chunk_agg<N, K, M, S, RAG>(w, d, a.pw, ck, x, aL, aR);
-    nest_row_scan<N, WARP>(lp, c, sh, aL, aR, cL, cR, XL, XR);
-    nest_chunk_finish<N, K, M, S, RAG>(w, d, ck, x, cL, cR, [&](int dir) { return dir ? XR : XL; }, out);
-    if constexpr (MODE == NEST_ROW_PASS) nest_row_load<N, K, RAG, H>(a.B + row, a.half, start, ck.cnt, on, x);
+    nest_row_inverse<N, K, M, RAG, WARP>(lp, w, a, g, sh, edge, x, out);
+    if constexpr (MODE == NEST_ROW_PASS) nest_row_load<N, K, RAG, H>(a.B + row, a.half, start, cnt, g.on, x);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         if constexpr (MODE == NEST_ROW_PASS) x[H + k] = N::add(x[H + k], out[k]);
         else x[H + k] = out[k];
     }
-    nest_row_halo<N, K, M, S, RAG, WARP>(c, a.cut.nc, ck.cnt, edge + 2 * H * a.TL, a.TL, x);
-    nest_chunk_agg<N, K, M, S, RAG>(w, d, a.pw, ck, x, aL, aR);
-    nest_row_scan<N, WARP>(lp, c, sh, aL, aR, cL, cR, XL, XR);
-    nest_chunk_finish<N, K, M, S, RAG>(w, d, ck, x, cL, cR, [&](int dir) { return dir ? XR : XL; }, out);
+    nest_row_inverse<N, K, M, RAG, WARP>(lp, w, a, g, sh, edge + 2 * H * a.TL, x, out);
 
     if constexpr (MODE == NEST_ROW_COPY) {
-        if constexpr (N::W == 2) {
-#pragma unroll
-            for (int j = 0; j < K / 4; ++j)
-                if (on && (!RAG || 4 * j < ck.cnt)) {
-#pragma unroll
-                    for (int q = 0; q < 2; ++q)
-                        *reinterpret_cast<float4*>(a.w + row + q * a.half + start + 4 * j) =
-                            make_float4(N::get(out[4 * j], q), N::get(out[4 * j + 1], q), N::get(out[4 * j + 2], q),
-                                        N::get(out[4 * j + 3], q));
-                }
-        } else {
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-                if (on && (!RAG || k < ck.cnt)) a.w[row + start + k] = out[k];
-        }
+        if (g.on) nest_row_store<N, K, RAG>(a.w + row, a.half, start, cnt, [&](int k) { return out[k]; });
     } else {
         RedAcc<T> red{T(0), T(0)};
         const bool wall_row = a.fix && (line == 0 || line == a.nlines - 1);
@@ -380,7 +428,7 @@ nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
         if constexpr (N::W == 2) {
 #pragma unroll
             for (int j = 0; j < K / 4; ++j)
-                if (on && (!RAG || 4 * j < ck.cnt)) {
+                if (g.on) {
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         const int p = q * a.half + start + 4 * j;
@@ -398,7 +446,7 @@ nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
         } else {
 #pragma unroll
             for (int k = 0; k < K; ++k)
-                if (on && (!RAG || k < ck.cnt)) {
+                if (g.on && (!RAG || k < cnt)) {
                     const size_t i = row + start + k;
                     a.w[i] = put(out[k], a.E[i], a.w[i], start + k);
                 }
