@@ -415,9 +415,10 @@ molt_status molt_batch_set_schedule(molt_batch* batch, int grid_rows, int grid_c
  * M^{-1} P = X = D_x D_y + D_x D_z + D_y D_z - 2 D_x D_y D_z (X = D_x D_y in 2D, Eq.
  * CH_2D_Doperator1); the 2D fixed-point iteration of Sec. 5.1 then holds with X in place of
  * D_x D_y.  FP32 fields of nz * ny * nx floats, row-major with x fastest, periodic or Neumann
- * lines (the grid conventions of molt_grid_create per axis).  Each iteration is a sequence of
- * single line sweeps over the whole field (not fused).  Errors of these calls are reported by
- * molt_last_error(NULL). */
+ * lines (the grid conventions of molt_grid_create per axis).  With equal factors an iteration is one
+ * pass per axis, its loop on the device; with different factors, or lines that those passes do not
+ * take, it is a sequence of single line sweeps over the whole field.  Errors of these calls are
+ * reported by molt_last_error(NULL). */
 typedef struct molt_solver3d molt_solver3d;
 
 /* nx, ny in [M + 2, 1024] (the y lines run as a batch of nz slabs, molt_batch_create), nz in

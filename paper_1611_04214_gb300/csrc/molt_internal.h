@@ -160,11 +160,11 @@ cudaError_t sweep(int axis, const LineParams<T>& lp, int kind, const OpArgs<T>& 
 // profile slots: the iteration's passes, the rhs inverse
 constexpr int kProfNestRows = 7, kProfNestCols = 24, kProfNestRowsRhs = 15, kProfNestColsRhs = 25;
 // What a nested column pass computes (nest.cuh).
-enum NestColMode { NEST_SCALAR = 0, NEST_VCH = 1, NEST_Z3 = 2, NEST_COPY = 3 };
+enum NestColMode { NEST_SCALAR = 0, NEST_VCH = 1, NEST_Z3 = 2, NEST_COPY = 3, NEST_Y3 = 4 };
 enum NestRowMode { NEST_ROW_PASS = 0, NEST_ROW_COPY = 1 };
 template <typename T>
 struct NestCols {
-    const T *in0 = nullptr, *in1 = nullptr, *Y = nullptr;
+    const T *in0 = nullptr, *in1 = nullptr, *in2 = nullptr, *Y = nullptr;
     T *o0 = nullptr, *o1 = nullptr, *o2 = nullptr;
     long long ld = 0, slab = 0;    // distances of two nodes of a column and of two slabs of columns
     int ncols = 0, nslabs = 1;

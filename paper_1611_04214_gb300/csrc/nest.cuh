@@ -492,7 +492,8 @@ __device__ __forceinline__ unsigned long long nest_from_bits(unsigned long long 
 template <typename T>
 struct NestColArgs {
     const T* in0;
-    const T* in1;     // vector model: the second component
+    const T* in1;     // vector model: the second component; 3D y pass: b
+    const T* in2;     // 3D y pass: c
     const T* Y;
     T* o0;
     T* o1;
@@ -791,6 +792,8 @@ __host__ __device__ constexpr int nest_col_pitch() {
     return NA == 1 ? K + 1 : NA * K + M + 1;
 }
 
+template <int K, int M>
+__host__ __device__ constexpr int nest_col3_pitch() { return 3 * K + 2 * M + 1; }
 
 // FORM 0: every chunk of every block has K nodes and the blocks' chunks come in multiples of 16; 1: chunks
 // of K nodes; 2: chunks of K and K - 1 nodes.
@@ -1014,6 +1017,172 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
                     return N::fma(nb, out[k], MODE == NEST_Z3 ? arr(0, k) : N::mul(N::splat(T(-2)), arr(0, k)));
                 });
             }
+        }
+    }
+    if (a.C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// =========================================================================================
+// 3D y pass (solver3d.cpp): from the z pass's a, b, c of one slab's columns
+//   E = Y - H H a,   B = H (-2a + H b),   A = -a + H (b + H c),
+// the data of the x pass w + E + H (B + H A).  Three fields through the two inverses of the kernel above; bound
+// like it by issue slots and barriers (1.75 of 4 instructions a cycle): 256^3 FP32 182 us = 2580 GB/s of its 28 B a
+// point; the z pass (16 B) 120 us, the x pass (20 B) 69 us.  The iteration takes 378 us; fifteen separate sweeps took 1817.
+// =========================================================================================
+template <class N, int M, int FORM, bool WIDE>
+__global__ void __launch_bounds__(256, 2)
+nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
+                  const __grid_constant__ NestCoef<typename N::V> w,
+                  const __grid_constant__ NestColArgs<typename N::T> a) {
+    using V = typename N::V;
+    using T = typename N::T;
+    constexpr bool RAG = FORM == 2;
+    constexpr int K = kNestColK, H = M / 2, S = 1, NF = 3, PITCH = nest_col3_pitch<K, M>();
+    // per thread: three arrays of the chunk's nodes, then the ends of the windows of fields 1 and 2
+    extern __shared__ __align__(16) unsigned char nest_sm[];
+    __shared__ NestColShared<N, NF> sh;
+    NestChunk ck;
+    const NestColGeo g = nest_col_geo<N, K, S, RAG>(lp, a, ck);
+    const V* all = reinterpret_cast<const V*>(nest_sm);
+    V* own = reinterpret_cast<V*>(nest_sm) + threadIdx.x * PITCH;
+    auto arr = [&](int f, int k) -> V& { return own[f * K + k]; };
+    auto end = [&](int q, int h) -> V& { return own[NF * K + (q - 1) * M + h]; };
+    V x[K + M], hl[H], hr[H];   // hl, hr: the window's ends of field 0
+    auto keep_ends = [&](int q, const V (&l)[H], const V (&r)[H]) {
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            if (q == 0) {
+                hl[h] = l[h];
+                hr[h] = r[h];
+            } else {
+                end(q, h) = l[h];
+                end(q, H + h) = r[h];
+            }
+        }
+    };
+    auto window_ends = [&](int q) {
+        V l[H], r[H];
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            l[h] = x[h];
+            r[h] = x[H + K + h];
+        }
+        keep_ends(q, l, r);
+    };
+    auto window = [&](int q) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) x[H + k] = arr(q, k);
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            x[h] = q == 0 ? hl[h] : end(q, h);
+            x[H + K + h] = q == 0 ? hr[h] : end(q, H + h);
+        }
+    };
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+        nest_col_window<N, K, M, RAG, WIDE>(q == 0 ? a.in0 : q == 1 ? a.in1 : a.in2, g, lp.n, lp.bc == BC_PERIODIC, a.ld, x);
+#pragma unroll
+        for (int k = 0; k < K; ++k) arr(q, k) = x[H + k];
+        window_ends(q);
+    }
+    V* ex = reinterpret_cast<V*>(nest_sm) + PITCH * g.nt;
+    T* dec = reinterpret_cast<T*>(ex + ((2 * NF) << a.lcp) * (a.slots + 4)) + threadIdx.x;
+    const NestColScan<V, T> c = nest_col_scan_setup<N, K, S, RAG>(lp, a, g, ck, ex, dec, sh);
+
+#pragma unroll 1
+    for (int level = 0; level < 2; ++level) {
+        if (level == 1) {
+            // edges of the chunks before and after this one (wrapped on periodic columns); as nest_cols_kernel
+            if (a.C > 1) nest_cluster_sync();
+            else __syncthreads();
+            const int nc = a.cut.nc, last = (nc - 1) - a.slots * (a.C - 1);
+            const bool pin = g.slot > 0, fin = g.slot < a.slots - 1 && g.ci < nc - 1;
+            const int pr = pin || !g.live ? g.rank : g.rank > 0 ? g.rank - 1 : a.C - 1;
+            const int fr = fin || !g.live ? g.rank : g.ci < nc - 1 ? g.rank + 1 : 0;
+            const int ps = pin ? g.slot - 1 : g.rank > 0 ? a.slots - 1 : last, fs = fin ? g.slot + 1 : 0;
+            const int pcnt = (!RAG || (g.ci > 0 ? g.ci - 1 : nc - 1) < a.cut.rem) ? K : K - S;
+            const V* pe = all + ((ps << a.lcp) + g.cpi) * PITCH + (pcnt - H);
+            const V* fe = all + ((fs << a.lcp) + g.cpi) * PITCH;
+#pragma unroll
+            for (int q = 0; q < NF; ++q) {
+                V l[H], r[H];
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const V *lq = pe + q * K + h, *rq = fe + q * K + h;
+                    l[h] = pr == g.rank ? *lq : nest_from_bits(nest_ld_cluster(lq, pr), V());
+                    r[h] = fr == g.rank ? *rq : nest_from_bits(nest_ld_cluster(rq, fr), V());
+                }
+                if (RAG && ck.cnt == K - S) {
+                    arr(q, K - 1) = r[0];
+#pragma unroll
+                    for (int h = 0; h + 1 < H; ++h) r[h] = r[h + 1];
+                }
+                keep_ends(q, l, r);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NF; ++q) {
+            window(q);
+            V aL, aR;
+            nest_chunk_agg<N, K, M, S, RAG>(lp, w, a.pw, ck, x, aL, aR);
+            if (g.slot < a.slots) {
+                V* e = ex + 2 * ((q << a.lcp) + g.cpi) * (a.slots + 4) + g.slot;
+                e[0] = aL;
+                e[a.slots + 4] = aR;
+            }
+            if (kNestGhosts<N, M> && (ck.mA | ck.mB)) {   // the ghosts
+                window_ends(q);
+                if (RAG) arr(q, K - 1) = x[H + K - 1];
+            }
+        }
+        // offset of the chunk in the fields (opaque: its addresses are not to be kept through the loop)
+        long long o0 = g.base + static_cast<long long>(g.start) * a.ld;
+        asm volatile("" : "+l"(o0));
+        nest_col_scan<N, NF, FORM == 0>(lp, c, sh, level);
+        // no block leaves while another may still read its shared memory
+        if (level == 1 && a.C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        V out[K];
+        auto finish = [&](int q) {
+            window(q);
+            nest_chunk_finish<N, K, M, S, RAG>(lp, w, ck, x, nest_col_carry<N, NF>(lp, c, sh, q, 0),
+                                               nest_col_carry<N, NF>(lp, c, sh, q, 1),
+                                               [&](int dir) { return nest_col_end<N, NF>(lp, c, sh, q, dir); }, out);
+        };
+        const V m1 = N::splat(T(-1)), m2 = N::splat(T(-2));
+        if (level == 0) {
+            finish(2);
+#pragma unroll
+            for (int k = 0; k < K; ++k) arr(2, k) = N::add(out[k], arr(1, k));              // b + H c
+            finish(1);
+#pragma unroll
+            for (int k = 0; k < K; ++k) arr(1, k) = N::fma(m2, arr(0, k), out[k]);          // -2a + H b
+            finish(0);
+#pragma unroll
+            for (int k = 0; k < K; ++k) arr(0, k) = out[k];
+        } else {
+            // out -> field f, or (other) other + s out
+            auto put = [&](T* f, const T* other, V so, V sf) {
+                if (!g.on) return;
+                V y[K];
+                if (other) {
+#pragma unroll
+                    for (int k = 0; k < K; ++k)
+                        if (!RAG || k < K - 1 || ck.cnt == K)
+                            y[k] = nest_load<N, WIDE>(other + o0 + static_cast<long long>(a.ld) * k, g.both);
+                }
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    if (!RAG || k < K - 1 || ck.cnt == K)
+                        nest_store<N, WIDE>(f + o0 + static_cast<long long>(a.ld) * k,
+                                            other ? N::fma(sf, y[k], N::mul(so, out[k])) : out[k], g.both);
+            };
+            const V one = N::splat(T(1));
+            finish(0);
+            put(a.o2, a.Y, m1, one);
+            finish(1);
+            put(a.o1, nullptr, one, one);
+            finish(2);
+            put(a.o0, a.in0, one, m1);
         }
     }
     if (a.C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

@@ -55,7 +55,7 @@ template <class F, int M, typename T>
 cudaError_t nest_cols_run(const LineParams<T>& lp, const NestCols<T>& p, cudaStream_t st, Prof* prof) {
     using N = NestVec<T, sizeof(T) == 4 ? 2 : 1>;
     NestColArgs<T> a{};
-    a.in0 = p.in0, a.in1 = p.in1, a.Y = p.Y, a.o0 = p.o0, a.o1 = p.o1, a.o2 = p.o2;
+    a.in0 = p.in0, a.in1 = p.in1, a.in2 = p.in2, a.Y = p.Y, a.o0 = p.o0, a.o1 = p.o1, a.o2 = p.o2;
     a.ld = static_cast<int>(p.ld), a.slab = p.slab, a.ncols = p.ncols;
     a.g1 = p.g1, a.beta = p.beta, a.vs = p.vs, a.comp = p.comp;
     int strips;
@@ -96,6 +96,10 @@ template <typename T, int M, int FORM, bool WIDE, int MODE> struct NestColsPass 
     static constexpr int kPitch = nest_col_pitch<kNestColK, M, MODE == NEST_COPY ? 1 : 3>();
     static constexpr int kNF = MODE == NEST_COPY ? 1 : 2, kSlot = MODE == NEST_COPY ? kProfNestColsRhs : kProfNestCols;
     static auto kern() { return nest_cols_kernel<NestVec<T, sizeof(T) == 4 ? 2 : 1>, M, FORM, WIDE, MODE>; }
+};
+template <typename T, int M, int FORM, bool WIDE> struct NestColsPass<T, M, FORM, WIDE, NEST_Y3> {
+    static constexpr int kPitch = nest_col3_pitch<kNestColK, M>(), kNF = 3, kSlot = kProfNestCols;
+    static auto kern() { return nest_cols3_kernel<NestVec<T, sizeof(T) == 4 ? 2 : 1>, M, FORM, WIDE>; }
 };
 
 // One row kernel, F::kern(); args has the layout but for `ahead`.
@@ -160,7 +164,7 @@ namespace detail {
 template <typename T, int M, int MODE>
 cudaError_t nest_cols_mode(const LineParams<T>& lp, const NestCols<T>& p, cudaStream_t st, Prof* prof) {
     bool wide = p.ncols % 2 == 0 && p.ld % 2 == 0 && p.slab % 2 == 0;
-    const T* fields[] = {p.in0, p.in1, p.Y, p.o0, p.o1, p.o2};
+    const T* fields[] = {p.in0, p.in1, p.in2, p.Y, p.o0, p.o1, p.o2};
     for (const T* f : fields) wide = wide && aligned8(f);
     const int nc = lp.n / kNestColK, C = (nc + 63) / 64;
     const int form = lp.n % kNestColK != 0 ? 2 : nc % (16 * C) != 0 ? 1 : 0;
@@ -182,6 +186,10 @@ cudaError_t nest_cols_m(const LineParams<T>& lp, int mode, const NestCols<T>& p,
         case NEST_SCALAR: return nest_cols_mode<T, M, NEST_SCALAR>(lp, p, st, prof);
         case NEST_VCH: return nest_cols_mode<T, M, NEST_VCH>(lp, p, st, prof);
         case NEST_COPY: return nest_cols_mode<T, M, NEST_COPY>(lp, p, st, prof);
+    }
+    if constexpr (sizeof(T) == 4) {   // 3D runs in FP32
+        if (mode == NEST_Z3) return nest_cols_mode<T, M, NEST_Z3>(lp, p, st, prof);
+        if (mode == NEST_Y3) return nest_cols_mode<T, M, NEST_Y3>(lp, p, st, prof);
     }
     return cudaErrorInvalidValue;
 }
