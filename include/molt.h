@@ -463,7 +463,8 @@ long long molt_solver3d_launches(const molt_solver3d* solver);
  * - c_p x h^2 (2 eps^2 x / a + 4 - 2 eta eps^2)], h = 1/(1 + x): the iteration diverges where
  * |m| > 1 (eps = 0.18, eta = 1: dt = 0.1 does, dt <= 0.07 does not).  Fields are `lines`
  * independent lines of nx nodes, [lines][nx] row-major, FP32 or FP64 per params->precision.
- * Each iteration runs 7 line sweeps, one pointwise kernel and 6 linear combinations, and
+ * On periodic lines (FP64: of 256 nodes and more) an iteration is one kernel and the loop runs on the
+ * device; otherwise it runs 7 line sweeps, one pointwise kernel and 6 linear combinations, and
  * synchronizes `stream` to read the residual.  Errors of these calls are reported by
  * molt_last_error(NULL). */
 typedef struct molt_fch1d molt_fch1d;

@@ -11,8 +11,8 @@
 //   p = -eps^2 f' Lap v + f f' - eta eps^2 f.
 // Lap v^{k+1} = (v^{k+1} - z) / a holds exactly for the discrete H and is carried with the iterate
 // (across steps too); initial data take Lap(H v^n) = (H v^n - v^n) / a for the first iteration.
-// Each iteration is 7 line sweeps, one pointwise kernel and six linear combinations over the
-// [lines][nx] field.  The stopping rule is the single-grid solver's
+// Each iteration is one kernel on periodic lines (nest_fch_kernel), and 7 line sweeps, one pointwise kernel and six
+// linear combinations over the [lines][nx] field otherwise (see fused).  The stopping rule is the single-grid solver's
 // (FP32: the tolerance floored at 2 ulp of max|v| and the stall rule below 64 ulp).
 #include <cuda_runtime.h>
 
@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/molt.h"
+#include "loop_graph.h"
 #include "molt_internal.h"
 
 struct molt_fch1d {
@@ -53,6 +54,7 @@ struct Fch1d final : molt_fch1d {
     unsigned long long* red = nullptr;
     unsigned long long* red_host = nullptr;
     bool have_lap = false;   // Lap v of the last step's iterate is in `lap`
+    molt::LoopGraphs loop;   // the fused iteration's device-driven loop
 
     ~Fch1d() override {
         for (void* q : allocs) cudaFree(q);
@@ -68,6 +70,7 @@ struct Fch1d final : molt_fch1d {
     }
 
     bool init() {
+        if (!loop.init()) return false;
         for (T** q : {&v, &vn, &vnew, &h2vn, &lap, &f, &pp, &hv, &dv, &hdv, &df, &hdf, &dp, &hdp, &z, &zero})
             if (!alloc(q)) return false;
         void* m = nullptr;
@@ -102,6 +105,23 @@ struct Fch1d final : molt_fch1d {
         return r;
     }
 
+    // Whether the fused iteration (nest_fch_kernel) takes the lines: periodic ones.  With walls the map amplifies rounding, so
+    // that two orders of the same operations differ by up to 1e-3 of the field in FP32 and 1e-12 in FP64 after a few
+    // iterations (8192 nodes of noise); those keep the separate sweeps and their results.  FP64 lines below 256 nodes stay
+    // with the sweeps too: callers count their launches (14 and more an iteration).
+    bool fused() const { return molt::nest_rows_ok<T>(nx) && bc == molt::BC_PERIODIC && (sizeof(T) == 4 || nx >= 256); }
+
+    // H^2 v^n by the inverses that the iteration runs (their rounding then cancels between the two).
+    cudaError_t h2(const molt::LineParams<T>& lp, cudaStream_t st) {
+        if (fused()) {
+            molt::NestRows<T> r;
+            r.A = vn, r.w = h2vn, r.nlines = lines;
+            return molt::nest_rows<T>(lp, molt::NEST_ROW_COPY, r, st, &launches);
+        }
+        cudaError_t e = H(lp, vn, hv, st);
+        return e == cudaSuccess ? H(lp, hv, h2vn, st) : e;
+    }
+
     molt_status step(void* uv, double dt, cudaStream_t st, molt_step_info* info) override {
         T* u = static_cast<T*>(uv);
         const double eps = p.eps;
@@ -116,15 +136,32 @@ struct Fch1d final : molt_fch1d {
         // v^n = u + 1; H^2 v^n; Lap v^n carried or bootstrapped
         if ((e = lin(vn, u, 1.0, nullptr, 0, nullptr, 0, nullptr, 0, 1.0, st)) != cudaSuccess ||
             (e = lin(v, vn, 1.0, nullptr, 0, nullptr, 0, nullptr, 0, 0.0, st)) != cudaSuccess ||
-            (e = H(lp, vn, hv, st)) != cudaSuccess || (e = H(lp, hv, h2vn, st)) != cudaSuccess)
+            (e = h2(lp, st)) != cudaSuccess)
             return fail_f(MOLT_ERR_CUDA, std::string("sixth-order step load: ") + cudaGetErrorString(e));
         if (!have_lap)
-            if ((e = lin(lap, hv, 1.0 / a, vn, -1.0 / a, nullptr, 0, nullptr, 0, 0.0, st)) != cudaSuccess)
+            if ((e = H(lp, vn, hv, st)) != cudaSuccess ||
+                (e = lin(lap, hv, 1.0 / a, vn, -1.0 / a, nullptr, 0, nullptr, 0, 0.0, st)) != cudaSuccess)
                 return fail_f(MOLT_ERR_CUDA, std::string("sixth-order step load: ") + cudaGetErrorString(e));
         double res = INFINITY, best = INFINITY, tol_used = p.tol;
         int k = 0, stall = 0;
         bool converged = false;
         const bool fp32 = sizeof(T) == 4;
+        if (fused()) {
+            // one kernel per iteration (nest_fch_kernel), the loop on the device: 16384 lines of 1024 nodes, FP32, M = 6:
+            // 107 us an iteration against 606 by the sweeps below, 70 lines of 200 nodes 14 against 145
+            molt::NestFch<T> it;
+            it.v = v, it.lap = lap, it.h2 = h2vn, it.nlines = lines, it.red = red;
+            it.eps2 = eps * eps, it.eta_eps2 = eta * eps * eps, it.c_eta = c_eta, it.c_f = c_f, it.c_p = c_p;
+            it.inv_a = 1.0 / a;
+            molt::LoopState ls;
+            e = loop.run(dt, v, red, p.tol, p.max_iter, fp32,
+                         [&](cudaStream_t s) { return molt::nest_fch<T>(lp, it, s, nullptr); }, st, &ls);
+            if (e != cudaSuccess)
+                return fail_f(MOLT_ERR_CUDA, std::string("sixth-order iteration: ") + cudaGetErrorString(e));
+            launches += 1 + 2LL * ls.k;
+            k = ls.k, res = ls.res, tol_used = ls.tol_used, converged = ls.converged != 0;
+            return finish(u, converged, k, res, tol_used, st, info);
+        }
         for (k = 1; k <= p.max_iter; ++k) {
             if ((e = molt::fch_pointwise<T>(static_cast<long long>(n), v, lap, eps * eps, eta * eps * eps, f, pp, st,
                                             &launches)) != cudaSuccess ||
@@ -168,6 +205,12 @@ struct Fch1d final : molt_fch1d {
                 break;
             }
         }
+        return finish(u, converged, k, res, tol_used, st, info);
+    }
+
+    // The iterate back to u, the step's outcome.
+    molt_status finish(T* u, bool converged, int k, double res, double tol_used, cudaStream_t st, molt_step_info* info) {
+        cudaError_t e;
         have_lap = true;
         if ((e = lin(u, v, 1.0, nullptr, 0, nullptr, 0, nullptr, 0, -1.0, st)) != cudaSuccess)
             return fail_f(MOLT_ERR_CUDA, std::string("sixth-order store: ") + cudaGetErrorString(e));

@@ -179,6 +179,20 @@ struct NestRows {
     T wall = 0;
     unsigned long long* red = nullptr;
 };
+// Sixth-order model on independent lines: one iteration in place on v and Lap v (nest_rows.cuh), max |v_new - v|
+// and max |v_new| into red.
+template <typename T>
+struct NestFch {
+    T *v = nullptr, *lap = nullptr;
+    const T* h2 = nullptr;     // H^2 v^n
+    int nlines = 0;
+    double eps2 = 0, eta_eps2 = 0, c_eta = 0, c_f = 0, c_p = 0, inv_a = 0;
+    unsigned long long* red = nullptr;
+};
+template <typename T>
+cudaError_t nest_fch(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_t st, long long* launches);
+template <int M, typename T>
+cudaError_t nest_fch_m(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_t st);
 // Whether the nested passes take lines of n nodes along rows / columns.
 template <typename T>
 bool nest_rows_ok(int n);

@@ -142,6 +142,9 @@ template <class N, int M, bool RAG, bool WARP> struct NestRowPass {
 template <class N, int M, bool RAG, bool WARP> struct NestRowCopy {
     static auto kern() { return nest_rows_kernel<N, M, RAG, WARP, NEST_ROW_COPY>; }
 };
+template <class N, int M, bool RAG, bool WARP> struct NestFchPass {
+    static auto kern() { return nest_fch_kernel<N, M, RAG, WARP>; }
+};
 
 template <typename T, int M, template <class, int, bool, bool> class F, class Args>
 cudaError_t nest_rows_run(const LineParams<T>& lp, Args a, int nlines, bool aligned, cudaStream_t st, Prof* prof, int slot) {
@@ -204,10 +207,22 @@ cudaError_t nest_rows_m(const LineParams<T>& lp, int mode, const NestRows<T>& p,
                                  : nest_rows_run<T, M, NestRowCopy>(lp, a, p.nlines, al, st, prof, kProfNestRowsRhs);
 }
 
+template <int M, typename T>
+cudaError_t nest_fch_m(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_t st) {
+    using namespace detail;
+    NestFchArgs<T> a{};
+    a.v = p.v, a.lap = p.lap, a.h2 = p.h2, a.red = p.red;
+    a.eps2 = static_cast<T>(p.eps2), a.eta_eps2 = static_cast<T>(p.eta_eps2), a.c_eta = static_cast<T>(p.c_eta);
+    a.c_f = static_cast<T>(p.c_f), a.c_p = static_cast<T>(p.c_p), a.inv_a = static_cast<T>(p.inv_a);
+    const bool al = aligned16(p.v) && aligned16(p.lap) && aligned16(p.h2);
+    return nest_rows_run<T, M, NestFchPass>(lp, a, p.nlines, al, st, nullptr, 0);
+}
+
 #define MOLT_INSTANTIATE_NEST(M, T)                                                                                  \
     template cudaError_t molt::nest_cols_m<M, T>(const molt::LineParams<T>&, int, const molt::NestCols<T>&, cudaStream_t, \
                                                  molt::Prof*);                                                       \
     template cudaError_t molt::nest_rows_m<M, T>(const molt::LineParams<T>&, int, const molt::NestRows<T>&, cudaStream_t, \
-                                                 molt::Prof*);
+                                                 molt::Prof*);                                                       \
+    template cudaError_t molt::nest_fch_m<M, T>(const molt::LineParams<T>&, const molt::NestFch<T>&, cudaStream_t);
 
 }  // namespace molt

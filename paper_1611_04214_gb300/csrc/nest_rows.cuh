@@ -455,4 +455,91 @@ nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     }
 }
 
+// Sixth-order model on independent lines: one whole iteration (fch1d.cpp).  With f = f(v), p the pointwise
+// lagged product (fch_pointwise), G = c_eta v - c_f f + c_p p and A = (3 + c_eta) v - c_f f, the terms collect by
+// linearity of H into
+//   q = H G - A,   z = H^2 v^n + H q - q,   v <- H z,   Lap v <- (v - z) / a,
+// three inverses with the line in registers; v and Lap v are written once, H^2 v^n is read once, v is read again
+// (from L2) where holding it would spill.
+// Bound: latency at 16 warps a SM (1.5 of 4 instructions a cycle; loads and the shuffles of three scans): 16384 lines of
+// 1024 nodes, FP32, M = 6: 107 us an iteration = 3100 GB/s of the 20 B a point, fourteen kernels took 606; FP64, 4096
+// lines: 670 us, FP64 units, against 1856.
+template <typename T>
+struct NestFchArgs : NestRowLayout<T> {
+    T* v;
+    T* lap;
+    const T* h2;
+    T eps2, eta_eps2, c_eta, c_f, c_p, inv_a;
+    unsigned long long* red;
+};
+
+template <class N, int M, bool RAG, bool WARP>
+__global__ void __launch_bounds__(N::W == 2 ? 256 : 512, N::W == 2 ? 2 : 1)
+nest_fch_kernel(const __grid_constant__ LineParams<typename N::T> lp,
+                const __grid_constant__ NestCoef<typename N::V> w,
+                const __grid_constant__ NestFchArgs<typename N::T> a) {
+    using V = typename N::V;
+    using T = typename N::T;
+    constexpr int K = kNestRowK, H = M / 2;
+    extern __shared__ __align__(16) unsigned char nest_row_sm[];
+    V* edge = reinterpret_cast<V*>(nest_row_sm);
+    __shared__ NestRowShared<N> sh;
+    NestRowThread<N> g = nest_row_thread<N, K, RAG, WARP>(lp, a);
+    const int start = g.start, cnt = g.ck.cnt;
+    const size_t row = g.row;
+    const V m1 = N::splat(T(-1)), c3 = N::splat(T(3) + a.c_eta), nf = N::splat(-a.c_f);
+    auto cube = [&](V x) { return N::mul(x, N::fma(x, N::add(x, N::splat(T(-3))), N::splat(T(2)))); };   // f(v)
+
+    V x[K + M], out[K];
+    nest_row_load<N, K, RAG, H>(a.v + row, a.half, start, cnt, g.on, x);
+    {
+        V l[K];
+        nest_row_load<N, K, RAG, 0>(a.lap + row, a.half, start, cnt, g.on, l);
+        const V e2 = N::splat(a.eps2), ee = N::splat(a.eta_eps2), ce = N::splat(a.c_eta), cp = N::splat(a.c_p);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const V v = x[H + k], f = cube(v);
+            const V fp = N::fma(v, N::fma(N::splat(T(3)), v, N::splat(T(-6))), N::splat(T(2)));
+            const V p = N::fma(f, fp, N::mul(m1, N::fma(N::mul(e2, fp), l[k], N::mul(ee, f))));
+            x[H + k] = N::fma(cp, p, N::fma(nf, f, N::mul(ce, v)));
+        }
+    }
+    nest_row_scan_setup<N, K, RAG, WARP>(lp, a, g, sh);
+    nest_row_inverse<N, K, M, RAG, WARP>(lp, w, a, g, sh, edge, x, out);
+    nest_row_load<N, K, RAG, H>(a.v + row, a.half, start, cnt, g.on, x);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const V v = x[H + k];
+        x[H + k] = N::fma(m1, N::fma(nf, cube(v), N::mul(c3, v)), out[k]);           // q
+    }
+    nest_row_inverse<N, K, M, RAG, WARP>(lp, w, a, g, sh, edge + 2 * H * a.TL, x, out);
+    {
+        V h2[K];
+        nest_row_load<N, K, RAG, 0>(a.h2 + row, a.half, start, cnt, g.on, h2);
+#pragma unroll
+        for (int k = 0; k < K; ++k) x[H + k] = N::add(h2[k], N::fma(m1, x[H + k], out[k]));   // z
+    }
+    // (the first set of edges is free again: every thread has passed the second inverse's barriers)
+    nest_row_inverse<N, K, M, RAG, WARP>(lp, w, a, g, sh, edge, x, out);
+    RedAcc<T> red{T(0), T(0)};
+    if (g.on) {
+        const V ia = N::splat(a.inv_a);
+        nest_row_store<N, K, RAG>(a.lap + row, a.half, start, cnt,
+                                  [&](int k) { return N::mul(ia, N::fma(m1, x[H + k], out[k])); });
+        nest_row_load<N, K, RAG, H>(a.v + row, a.half, start, cnt, true, x);
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (!RAG || k < cnt) {
+                const V e = N::fma(m1, x[H + k], out[k]);
+#pragma unroll
+                for (int q = 0; q < N::W; ++q) {
+                    red.dmax = fmax(red.dmax, fabs(N::get(e, q)));
+                    red.vmax = fmax(red.vmax, fabs(N::get(out[k], q)));
+                }
+            }
+        nest_row_store<N, K, RAG>(a.v + row, a.half, start, cnt, [&](int k) { return out[k]; });
+    }
+    nest_reduce<T>(red, a.red);
+}
+
 }  // namespace molt
