@@ -238,6 +238,25 @@ cudaError_t loop_init(LoopState* ls, unsigned long long* red, cudaStream_t st);
 cudaError_t loop_check(cudaGraphConditionalHandle h, LoopState* ls, unsigned long long* red, double tol,
                        int max_iter, int fp32, cudaStream_t st);
 
+// A single 1D line: the whole fixed-point loop of a stage in one block (nest_line.cuh), the outcome in *ls.
+template <typename T>
+struct NestLine {
+    T* w = nullptr;          // the iterate, in place
+    const T* Y = nullptr;    // the stage's right side, or r with Y = H_o H_i r
+    const T* r = nullptr;
+    T* Yout = nullptr;       // only compute Y from r, into here
+    T g2 = 0, g1 = 0, beta = 0, wall = 0;
+    int fix = 0;             // Dirichlet lines: `wall` on the walls after every iteration
+    double tol = 0;
+    int max_iter = 0;
+    LoopState* ls = nullptr;
+};
+template <typename T>
+bool nest_line_ok(int n);
+template <typename T>
+cudaError_t nest_line(const LineParams<T>& li, const LineParams<T>& lo, const NestLine<T>& p, cudaStream_t st,
+                      long long* launches);
+
 // y[j][i] += sum_k a[k][j] b[k][i] (k < terms <= 4), the sum in FP64, for a [ny][nx] field.
 struct Separable {
     const double* a[4];

@@ -10,7 +10,7 @@
 //
 // Stage solve (v - tau F(v) = r):  parameters from the regime switch of Sec. 3.1.2 (with
 // dt -> tau as in Sec. 4.1-4.2), inner factor = larger c.
-//   1D:  w <- H_o[ H_i[r + beta G(w)] - beta G(w) ]                     (2 sweeps)
+//   1D:  w <- H_o[ H_i[r + beta G(w)] - beta G(w) ]   (2 sweeps; up to 4096 nodes one kernel is the whole loop, nest_line.cuh)
 //   2D:  Y = H_ox H_oy H_ix H_iy r once, then per iteration
 //        (y, c_i)  T = H_iy G(w),  S = H_iy w
 //        (x, c_i)  U = S + H_ix(w - S),  P = beta (H_ix(2T - G) - T) + U
@@ -801,6 +801,37 @@ struct Solver final : molt_solver {
         return &lg;
     }
 
+    // A stage of a single line: one kernel runs the whole loop (both execution modes).
+    molt_status line_stage(const Passes& ps, const StageParams& sp, const T* rhs, bool y_given, cudaStream_t st, int* iters,
+                           double* res_out, double* tol_out) {
+        cudaError_t e;
+        molt::NestLine<T> a;
+        a.w = w, a.g2 = ps.g2, a.g1 = ps.g1, a.beta = ps.beta;
+        a.tol = p.tol, a.max_iter = p.max_iter, a.ls = ls;
+        if (bc == molt::BC_DIRICHLET) {
+            // Y by the loop's own inverses: their rounding (of d above all) cancels between Y and the iteration
+            if (!y_given) {
+                a.r = rhs, a.Yout = Y;
+                if ((e = molt::nest_line<T>(ps.lix, ps.lox, a, st, &launches)) != cudaSuccess)
+                    return cuda_fail(e, "rhs inverse");
+                a.Yout = nullptr;
+            }
+            if ((e = add_dirichlet_offset(sp, Y, st)) != cudaSuccess) return cuda_fail(e, "Dirichlet offset");
+            a.fix = 1, a.wall = T(-1);
+            y_given = true;
+        }
+        a.Y = y_given ? Y : nullptr;
+        a.r = rhs;
+        if ((e = molt::nest_line<T>(ps.lix, ps.lox, a, st, &launches)) != cudaSuccess) return cuda_fail(e, "line stage");
+        if ((e = cudaMemcpyAsync(ls_host, ls, sizeof(molt::LoopState), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
+            return cuda_fail(e, "loop state copy");
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "stream sync");
+        *iters = ls_host->k;
+        *res_out = ls_host->res;
+        *tol_out = ls_host->tol_used;
+        return ls_host->converged ? MOLT_OK : MOLT_ERR_NOT_CONVERGED;
+    }
+
     // Solve v - tau F(v) = r for w (in: first guess, out: last iterate), r in stored form.
     // With y_given, the field Y already holds M_o^{-1} M_i^{-1} r and rhs is not read.
     // With `given`, its passes are run (the vector CH stage) and Y must be given.
@@ -811,6 +842,8 @@ struct Solver final : molt_solver {
         if (given) ps = *given;
         else if (!make_passes(sp, &ps)) return MOLT_ERR_ARG;
         cudaError_t e = cudaSuccess;
+        if (g.dim == 1 && !given && molt::nest_line_ok<T>(g.nx))
+            return line_stage(ps, sp, rhs, y_given, st, iters, res_out, tol_out);
         if (!y_given) {
             // Y = M_o^{-1} M_i^{-1} r
             if ((e = rhs_inverse(sp.c_in, sp.c_out, rhs, Y, st)) != cudaSuccess) return cuda_fail(e, "rhs inverse");
