@@ -736,13 +736,12 @@ def fch1d_leg():
 
 FCH2D = dict(name="fch2d_4096_be_periodic", n=4096, eps=0.18, eta=1.0, dt=0.05, M=6, amp=0.05, seed=0, iters=10,
              steps=3)
-# per 2D sixth-order iteration (the regrouped form), in values per point: the pointwise kernel 4,
-# 14 one-field sweeps 28, eleven linear combinations 4 + 3 + 4 + 3 + 5 + 3 + 3 + 5 + 3 + 4 + 5 = 42,
-# the residual 2 and, in FP32, max|v| 1; per step: v^n 2, M^{-2} v^n 8, v, Lap v and X W of W 15,
-# the store 2
-FCH2D_VALUES_ITER = {"fp32": 4 + 28 + 42 + 2 + 1, "fp64": 4 + 28 + 42 + 2}
-FCH2D_VALUES_STEP = 2 + 8 + 15 + 2
-FCH2D_SWEEPS_ITER, FCH2D_SWEEPS_STEP = 14, 7
+# per 2D sixth-order iteration (periodic: collected axis by axis), in values per point: the y pass of three fields
+# reads 5 and writes 3, the x pass reads 4 and writes 1, H_y W 2, v and the next fields read 4 and write 6; per step:
+# v^n 2, M^{-2} v^n 4, H_y W 2, v and the fields 10, the store 2
+FCH2D_VALUES_ITER = {"fp32": 8 + 5 + 2 + 10, "fp64": 8 + 5 + 2 + 10}
+FCH2D_VALUES_STEP = 2 + 4 + 2 + 10 + 2
+FCH2D_SWEEPS_ITER, FCH2D_SWEEPS_STEP = 11, 7
 
 
 def fch2d_leg():

@@ -497,9 +497,10 @@ long long molt_fch1d_launches(const molt_fch1d* solver);
  *        + (3X - 3X^2 + X^3) W,
  * so that Lap v = K W / a exactly (the first step starts from W = v^n; later steps carry W).
  * Fields [ny][nx] row-major, x fastest, FP32 or FP64 per params->precision, periodic or Neumann
- * (the grid conventions of molt_grid_create).  Regrouped by linearity, each iteration runs 14
- * one-field line sweeps, one pointwise kernel and 11 linear combinations, and synchronizes
- * `stream` to read the residual.
+ * (the grid conventions of molt_grid_create).  On periodic grids an iteration is four kernels (the
+ * terms collected axis by axis) and the loop runs on the device.  Otherwise, regrouped by
+ * linearity, each iteration runs 14 one-field line sweeps, one pointwise kernel and 11 linear
+ * combinations, and synchronizes `stream` to read the residual.
  * Errors are reported by molt_last_error(NULL). */
 typedef struct molt_fch2d molt_fch2d;
 

@@ -160,16 +160,17 @@ cudaError_t sweep(int axis, const LineParams<T>& lp, int kind, const OpArgs<T>& 
 // profile slots: the iteration's passes, the rhs inverse
 constexpr int kProfNestRows = 7, kProfNestCols = 24, kProfNestRowsRhs = 15, kProfNestColsRhs = 25;
 // What a nested column pass computes (nest.cuh).
-enum NestColMode { NEST_SCALAR = 0, NEST_VCH = 1, NEST_Z3 = 2, NEST_COPY = 3, NEST_Y3 = 4 };
+enum NestColMode { NEST_SCALAR = 0, NEST_VCH = 1, NEST_Z3 = 2, NEST_COPY = 3, NEST_Y3 = 4, NEST_FCH2 = 5 };
 enum NestRowMode { NEST_ROW_PASS = 0, NEST_ROW_COPY = 1 };
 template <typename T>
 struct NestCols {
-    const T *in0 = nullptr, *in1 = nullptr, *in2 = nullptr, *Y = nullptr;
+    const T *in0 = nullptr, *in1 = nullptr, *in2 = nullptr, *Y = nullptr, *U = nullptr;
     T *o0 = nullptr, *o1 = nullptr, *o2 = nullptr;
     long long ld = 0, slab = 0;    // distances of two nodes of a column and of two slabs of columns
     int ncols = 0, nslabs = 1;
     T g1 = 0, beta = 0, vs = 0;
     int comp = 0;
+    int single = 0;                // copy: one inverse instead of two
 };
 template <typename T>
 struct NestRows {
@@ -193,6 +194,20 @@ template <typename T>
 cudaError_t nest_fch(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_t st, long long* launches);
 template <int M, typename T>
 cudaError_t nest_fch_m(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_t st);
+// Sixth-order model in 2D: the x pass that opens an iteration (nest_rows.cuh): v from W and hy = H_y W, the fields
+// p, q, r, u, z of the y pass (NEST_FCH2: in0 .. in2 = p, q, r, U = u, Y = z), max |v_new - v| and max |v_new| into red.
+template <typename T>
+struct NestFch2 {
+    const T *W = nullptr, *hy = nullptr, *m2 = nullptr;
+    T *v = nullptr, *p = nullptr, *q = nullptr, *r = nullptr, *u = nullptr, *z = nullptr;
+    int nlines = 0;
+    double eps2 = 0, eta_eps2 = 0, c_eta = 0, c_f = 0, c_p = 0, inv_a = 0;
+    unsigned long long* red = nullptr;
+};
+template <typename T>
+cudaError_t nest_fch2(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_t st, long long* launches);
+template <int M, typename T>
+cudaError_t nest_fch2_m(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_t st);
 // Whether the nested passes take lines of n nodes along rows / columns.
 template <typename T>
 bool nest_rows_ok(int n);

@@ -71,13 +71,26 @@ cudaError_t nest_fch(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_t 
     return cudaErrorInvalidValue;
 }
 
+template <typename T>
+cudaError_t nest_fch2(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_t st, long long* launches) {
+    if (launches) *launches += 1;
+    const LineParams<T> q = nest_line_params(lp);
+    switch (lp.M) {
+        case 2: return nest_fch2_m<2, T>(q, p, st);
+        case 4: return nest_fch2_m<4, T>(q, p, st);
+        case 6: return nest_fch2_m<6, T>(q, p, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
 #define MOLT_NEST_ENTRY(T)                                                                                            \
     template LineParams<T> nest_line_params<T>(const LineParams<T>&);                                                \
     template bool nest_rows_ok<T>(int);                                                                              \
     template bool nest_cols_ok<T>(int);                                                                              \
     template cudaError_t nest_cols<T>(const LineParams<T>&, int, const NestCols<T>&, cudaStream_t, long long*, Prof*); \
     template cudaError_t nest_rows<T>(const LineParams<T>&, int, const NestRows<T>&, cudaStream_t, long long*, Prof*);    \
-    template cudaError_t nest_fch<T>(const LineParams<T>&, const NestFch<T>&, cudaStream_t, long long*);
+    template cudaError_t nest_fch<T>(const LineParams<T>&, const NestFch<T>&, cudaStream_t, long long*);                  \
+    template cudaError_t nest_fch2<T>(const LineParams<T>&, const NestFch2<T>&, cudaStream_t, long long*);
 MOLT_NEST_ENTRY(float)
 MOLT_NEST_ENTRY(double)
 

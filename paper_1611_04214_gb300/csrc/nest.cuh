@@ -482,7 +482,7 @@ __device__ __forceinline__ unsigned long long nest_from_bits(unsigned long long 
 //       A = beta (2a - b) - w + 2s - t,  B = -beta a - 2 (s - t),  E = Y - t,
 //     the y part of the iteration whose x part is w + E + H (B + H A) (solver.cpp);
 //   3D z pass:  outputs a3 = t, b3 = -2s + 4t - beta a, c3 = -w + 4s - 4t + beta (3a - b);
-//   copy: out = H H in.
+//   copy: out = H H in, or H in.
 // Bound: issue slots and the latency of the scan's barriers (1.5 to 1.9 of 4 instructions a cycle, 16 warps a SM), not
 // memory: 4096^2 Neumann FP32 198 us = 1700 GB/s of its 20 B a point, the row pass 80 us.  Two blocks a SM with 128
 // registers, chunks of K = 8: 4096^2 Neumann FP32 276 us an iteration, vector model 593, 2048^2 78, 1001 x 777 37;
@@ -495,6 +495,7 @@ struct NestColArgs {
     const T* in1;     // vector model: the second component; 3D y pass: b
     const T* in2;     // 3D y pass: c
     const T* Y;
+    const T* U;       // sixth-order pass: u
     T* o0;
     T* o1;
     T* o2;
@@ -507,6 +508,7 @@ struct NestColArgs {
     NestCut cut;
     T g1, beta, vs;
     int comp;
+    int single;       // copy: one inverse only
     NestPow<T> pw;
     int exact;        // the boundary solve is needed (see nest_col_scan)
 };
@@ -875,8 +877,8 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     const NestColScan<V, T> c = nest_col_scan_setup<N, K, S, RAG>(lp, a, g, ck, ex, dec, sh);
 
 #pragma unroll 1
-    for (int level = 0; level < 2; ++level) {
-        if (level == 1) {
+    for (int level = MODE == NEST_COPY && a.single ? 1 : 0; level < 2; ++level) {
+        if (level == 1 && !(MODE == NEST_COPY && a.single)) {
             // edges of the chunks before and after this one (wrapped on periodic columns)
             if (a.C > 1) nest_cluster_sync();
             else __syncthreads();
@@ -1028,8 +1030,11 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
 // the data of the x pass w + E + H (B + H A).  Three fields through the two inverses of the kernel above; bound
 // like it by issue slots and barriers (1.75 of 4 instructions a cycle): 256^3 FP32 182 us = 2580 GB/s of its 28 B a
 // point; the z pass (16 B) 120 us, the x pass (20 B) 69 us.  The iteration takes 378 us; fifteen separate sweeps took 1817.
+// Sixth-order model (fch2d.cpp), the same kernel with the fields p, q, r, u and z of nest_fch2_kernel:
+//   E = z + H (u + H p),   B = u + H (2p - u + H q),   A = p + H (q + H r):
+// 2048^2 FP32, M = 6: 97 us = 1380 GB/s of its 32 B a point, 1.07 of 4 instructions a cycle (clusters of four blocks).
 // =========================================================================================
-template <class N, int M, int FORM, bool WIDE>
+template <class N, int M, int FORM, bool WIDE, int MODE>
 __global__ void __launch_bounds__(256, 2)
 nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
                   const __grid_constant__ NestCoef<typename N::V> w,
@@ -1150,15 +1155,21 @@ nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
         };
         const V m1 = N::splat(T(-1)), m2 = N::splat(T(-2));
         if (level == 0) {
+            constexpr bool SIX = MODE == NEST_FCH2;
+            auto u = [&](int k) {   // (a register array of it would spill)
+                return g.on && (!RAG || k < K - 1 || ck.cnt == K)
+                           ? nest_load<N, WIDE>(a.U + o0 + static_cast<long long>(a.ld) * k, g.both) : N::zero();
+            };
             finish(2);
 #pragma unroll
             for (int k = 0; k < K; ++k) arr(2, k) = N::add(out[k], arr(1, k));              // b + H c
             finish(1);
 #pragma unroll
-            for (int k = 0; k < K; ++k) arr(1, k) = N::fma(m2, arr(0, k), out[k]);          // -2a + H b
+            for (int k = 0; k < K; ++k)                                                     // -2a + H b
+                arr(1, k) = SIX ? N::fma(N::splat(T(2)), arr(0, k), N::fma(m1, u(k), out[k])) : N::fma(m2, arr(0, k), out[k]);
             finish(0);
 #pragma unroll
-            for (int k = 0; k < K; ++k) arr(0, k) = out[k];
+            for (int k = 0; k < K; ++k) arr(0, k) = SIX ? N::add(u(k), out[k]) : out[k];
         } else {
             // out -> field f, or (other) other + s out
             auto put = [&](T* f, const T* other, V so, V sf) {
@@ -1178,11 +1189,11 @@ nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
             };
             const V one = N::splat(T(1));
             finish(0);
-            put(a.o2, a.Y, m1, one);
+            put(a.o2, a.Y, MODE == NEST_FCH2 ? one : m1, one);
             finish(1);
-            put(a.o1, nullptr, one, one);
+            put(a.o1, MODE == NEST_FCH2 ? a.U : nullptr, one, one);
             finish(2);
-            put(a.o0, a.in0, one, m1);
+            put(a.o0, a.in0, one, MODE == NEST_FCH2 ? one : m1);
         }
     }
     if (a.C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

@@ -55,7 +55,7 @@ template <class F, int M, typename T>
 cudaError_t nest_cols_run(const LineParams<T>& lp, const NestCols<T>& p, cudaStream_t st, Prof* prof) {
     using N = NestVec<T, sizeof(T) == 4 ? 2 : 1>;
     NestColArgs<T> a{};
-    a.in0 = p.in0, a.in1 = p.in1, a.in2 = p.in2, a.Y = p.Y, a.o0 = p.o0, a.o1 = p.o1, a.o2 = p.o2;
+    a.in0 = p.in0, a.in1 = p.in1, a.in2 = p.in2, a.Y = p.Y, a.U = p.U, a.single = p.single, a.o0 = p.o0, a.o1 = p.o1, a.o2 = p.o2;
     a.ld = static_cast<int>(p.ld), a.slab = p.slab, a.ncols = p.ncols;
     a.g1 = p.g1, a.beta = p.beta, a.vs = p.vs, a.comp = p.comp;
     int strips;
@@ -97,10 +97,14 @@ template <typename T, int M, int FORM, bool WIDE, int MODE> struct NestColsPass 
     static constexpr int kNF = MODE == NEST_COPY ? 1 : 2, kSlot = MODE == NEST_COPY ? kProfNestColsRhs : kProfNestCols;
     static auto kern() { return nest_cols_kernel<NestVec<T, sizeof(T) == 4 ? 2 : 1>, M, FORM, WIDE, MODE>; }
 };
-template <typename T, int M, int FORM, bool WIDE> struct NestColsPass<T, M, FORM, WIDE, NEST_Y3> {
+template <typename T, int M, int FORM, bool WIDE, int MODE> struct NestCols3Pass {
     static constexpr int kPitch = nest_col3_pitch<kNestColK, M>(), kNF = 3, kSlot = kProfNestCols;
-    static auto kern() { return nest_cols3_kernel<NestVec<T, sizeof(T) == 4 ? 2 : 1>, M, FORM, WIDE>; }
+    static auto kern() { return nest_cols3_kernel<NestVec<T, sizeof(T) == 4 ? 2 : 1>, M, FORM, WIDE, MODE>; }
 };
+template <typename T, int M, int FORM, bool WIDE>
+struct NestColsPass<T, M, FORM, WIDE, NEST_Y3> : NestCols3Pass<T, M, FORM, WIDE, NEST_Y3> {};
+template <typename T, int M, int FORM, bool WIDE>
+struct NestColsPass<T, M, FORM, WIDE, NEST_FCH2> : NestCols3Pass<T, M, FORM, WIDE, NEST_FCH2> {};
 
 // One row kernel, F::kern(); args has the layout but for `ahead`.
 template <class F, class N, int M, bool WARP, class Args>
@@ -146,6 +150,10 @@ template <class N, int M, bool RAG, bool WARP> struct NestFchPass {
     static auto kern() { return nest_fch_kernel<N, M, RAG, WARP>; }
 };
 
+template <class N, int M, bool RAG, bool WARP> struct NestFch2Pass {
+    static auto kern() { return nest_fch2_kernel<N, M, RAG, WARP>; }
+};
+
 template <typename T, int M, template <class, int, bool, bool> class F, class Args>
 cudaError_t nest_rows_run(const LineParams<T>& lp, Args a, int nlines, bool aligned, cudaStream_t st, Prof* prof, int slot) {
     int W;
@@ -167,7 +175,7 @@ namespace detail {
 template <typename T, int M, int MODE>
 cudaError_t nest_cols_mode(const LineParams<T>& lp, const NestCols<T>& p, cudaStream_t st, Prof* prof) {
     bool wide = p.ncols % 2 == 0 && p.ld % 2 == 0 && p.slab % 2 == 0;
-    const T* fields[] = {p.in0, p.in1, p.in2, p.Y, p.o0, p.o1, p.o2};
+    const T* fields[] = {p.in0, p.in1, p.in2, p.Y, p.U, p.o0, p.o1, p.o2};
     for (const T* f : fields) wide = wide && aligned8(f);
     const int nc = lp.n / kNestColK, C = (nc + 63) / 64;
     const int form = lp.n % kNestColK != 0 ? 2 : nc % (16 * C) != 0 ? 1 : 0;
@@ -189,6 +197,7 @@ cudaError_t nest_cols_m(const LineParams<T>& lp, int mode, const NestCols<T>& p,
         case NEST_SCALAR: return nest_cols_mode<T, M, NEST_SCALAR>(lp, p, st, prof);
         case NEST_VCH: return nest_cols_mode<T, M, NEST_VCH>(lp, p, st, prof);
         case NEST_COPY: return nest_cols_mode<T, M, NEST_COPY>(lp, p, st, prof);
+        case NEST_FCH2: return nest_cols_mode<T, M, NEST_FCH2>(lp, p, st, prof);
     }
     if constexpr (sizeof(T) == 4) {   // 3D runs in FP32
         if (mode == NEST_Z3) return nest_cols_mode<T, M, NEST_Z3>(lp, p, st, prof);
@@ -218,11 +227,25 @@ cudaError_t nest_fch_m(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_
     return nest_rows_run<T, M, NestFchPass>(lp, a, p.nlines, al, st, nullptr, 0);
 }
 
+template <int M, typename T>
+cudaError_t nest_fch2_m(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_t st) {
+    using namespace detail;
+    NestFch2Args<T> a{};
+    a.W = p.W, a.hy = p.hy, a.m2 = p.m2, a.v = p.v, a.p = p.p, a.q = p.q, a.r = p.r, a.u = p.u, a.z = p.z, a.red = p.red;
+    a.eps2 = static_cast<T>(p.eps2), a.eta_eps2 = static_cast<T>(p.eta_eps2), a.c_eta = static_cast<T>(p.c_eta);
+    a.c_f = static_cast<T>(p.c_f), a.c_p = static_cast<T>(p.c_p), a.inv_a = static_cast<T>(p.inv_a);
+    bool al = true;
+    const T* fields[] = {p.W, p.hy, p.m2, p.v, p.p, p.q, p.r, p.u, p.z};
+    for (const T* f : fields) al = al && aligned16(f);
+    return nest_rows_run<T, M, NestFch2Pass>(lp, a, p.nlines, al, st, nullptr, 0);
+}
+
 #define MOLT_INSTANTIATE_NEST(M, T)                                                                                  \
     template cudaError_t molt::nest_cols_m<M, T>(const molt::LineParams<T>&, int, const molt::NestCols<T>&, cudaStream_t, \
                                                  molt::Prof*);                                                       \
     template cudaError_t molt::nest_rows_m<M, T>(const molt::LineParams<T>&, int, const molt::NestRows<T>&, cudaStream_t, \
                                                  molt::Prof*);                                                       \
-    template cudaError_t molt::nest_fch_m<M, T>(const molt::LineParams<T>&, const molt::NestFch<T>&, cudaStream_t);
+    template cudaError_t molt::nest_fch_m<M, T>(const molt::LineParams<T>&, const molt::NestFch<T>&, cudaStream_t);      \
+    template cudaError_t molt::nest_fch2_m<M, T>(const molt::LineParams<T>&, const molt::NestFch2<T>&, cudaStream_t);
 
 }  // namespace molt

@@ -542,4 +542,126 @@ nest_fch_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     nest_reduce<T>(red, a.red);
 }
 
+// Four nodes 4j .. 4j + 3 of a thread's chunk.
+template <class N, bool RAG>
+__device__ __forceinline__ void nest_row_load4(const typename N::T* f, int half, int start, int cnt, int j,
+                                               typename N::V (&x)[4]) {
+    using T = typename N::T;
+    if constexpr (N::W == 2) {
+        const float4 lo = *reinterpret_cast<const float4*>(f + start + 4 * j);
+        const float4 hi = *reinterpret_cast<const float4*>(f + half + start + 4 * j);
+        x[0] = N::pair(lo.x, hi.x), x[1] = N::pair(lo.y, hi.y), x[2] = N::pair(lo.z, hi.z), x[3] = N::pair(lo.w, hi.w);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = !RAG || 4 * j + i < cnt ? f[start + 4 * j + i] : T(0);
+    }
+}
+template <class N, bool RAG>
+__device__ __forceinline__ void nest_row_store4(typename N::T* f, int half, int start, int cnt, int j,
+                                                const typename N::V (&x)[4]) {
+    if constexpr (N::W == 2) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            *reinterpret_cast<float4*>(f + q * half + start + 4 * j) =
+                make_float4(N::get(x[0], q), N::get(x[1], q), N::get(x[2], q), N::get(x[3], q));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (!RAG || 4 * j + i < cnt) f[start + 4 * j + i] = x[i];
+    }
+}
+
+// Sixth-order model in 2D, the x pass that opens an iteration (fch2d.cpp): from W and H_y W
+//   v = H_x H_y W,  X W = v - H_x W - H_y W + W,  a Lap v = 2v - H_x W - H_y W,
+// and from these, point by point, the fields of the y pass
+//   p = A + E,  q = -(s1 + 2p),  r = 2 s1 + E,  u = -E - X W,  z = M^{-2} v^n + X W - W
+// with s1 = 2A + B.  v goes out before the second inverse and is read again after it, so that one inverse's
+// registers are live at a time.
+// Bound: latency of two line chains at 16 warps a SM and 40 B a point: 2048^2 FP32, M = 6: 60 us = 2800 GB/s.  The whole
+// iteration (y pass 97, x pass 28, H_y W 22, this 60 us) takes 210 us; fourteen sweeps and twelve other kernels took 455.
+template <typename T>
+struct NestFch2Args : NestRowLayout<T> {
+    const T *W, *hy, *m2;
+    T *v, *p, *q, *r, *u, *z;
+    T eps2, eta_eps2, c_eta, c_f, c_p, inv_a;
+    unsigned long long* red;
+};
+
+template <class N, int M, bool RAG, bool WARP>
+__global__ void __launch_bounds__(N::W == 2 ? 256 : 512, N::W == 2 ? 2 : 1)
+nest_fch2_kernel(const __grid_constant__ LineParams<typename N::T> lp,
+                 const __grid_constant__ NestCoef<typename N::V> w,
+                 const __grid_constant__ NestFch2Args<typename N::T> a) {
+    using V = typename N::V;
+    using T = typename N::T;
+    constexpr int K = kNestRowK, H = M / 2;
+    extern __shared__ __align__(16) unsigned char nest_row_sm[];
+    V* edge = reinterpret_cast<V*>(nest_row_sm);
+    __shared__ NestRowShared<N> sh;
+    NestRowThread<N> g = nest_row_thread<N, K, RAG, WARP>(lp, a);
+    const int start = g.start, cnt = g.ck.cnt;
+    const size_t row = g.row;
+    const V m1 = N::splat(T(-1)), two = N::splat(T(2)), three = N::splat(T(3));
+    V x[K + M], out[K];
+    RedAcc<T> red{T(0), T(0)};
+    nest_row_load<N, K, RAG, H>(a.hy + row, a.half, start, cnt, g.on, x);
+    nest_row_scan_setup<N, K, RAG, WARP>(lp, a, g, sh);
+    nest_row_inverse<N, K, M, RAG, WARP>(lp, w, a, g, sh, edge, x, out);
+    if (g.on) {
+#pragma unroll
+        for (int j = 0; j < K / 4; ++j) {
+            V o[4];
+            nest_row_load4<N, RAG>(a.v + row, a.half, start, cnt, j, o);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (!RAG || 4 * j + i < cnt) {
+                    const V e = N::fma(m1, o[i], out[4 * j + i]);
+#pragma unroll
+                    for (int q = 0; q < N::W; ++q) {
+                        red.dmax = fmax(red.dmax, fabs(N::get(e, q)));
+                        red.vmax = fmax(red.vmax, fabs(N::get(out[4 * j + i], q)));
+                    }
+                }
+        }
+        nest_row_store<N, K, RAG>(a.v + row, a.half, start, cnt, [&](int k) { return out[k]; });
+    }
+    nest_row_load<N, K, RAG, H>(a.W + row, a.half, start, cnt, g.on, x);
+    nest_row_inverse<N, K, M, RAG, WARP>(lp, w, a, g, sh, edge + 2 * H * a.TL, x, out);
+    if (g.on) {
+        const V e2 = N::splat(a.eps2), ee = N::splat(a.eta_eps2), cp = N::splat(a.c_p), nf = N::splat(-a.c_f);
+        const V c3 = N::splat(T(3) + a.c_eta), c32 = N::splat(T(3) + T(2) * a.c_eta), nf2 = N::splat(T(-2) * a.c_f);
+        const V ia = N::splat(a.inv_a);
+#pragma unroll
+        for (int j = 0; j < K / 4; ++j) {
+            V v[4], hy[4], m2[4], P[4], Q[4], R[4], U[4];
+            nest_row_load4<N, RAG>(a.v + row, a.half, start, cnt, j, v);
+            nest_row_load4<N, RAG>(a.hy + row, a.half, start, cnt, j, hy);
+            nest_row_load4<N, RAG>(a.m2 + row, a.half, start, cnt, j, m2);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const V W = x[H + 4 * j + i], t = v[i];
+                const V h = N::add(out[4 * j + i], hy[i]);                              // H_x W + H_y W
+                const V lap = N::mul(ia, N::fma(two, t, N::mul(m1, h)));
+                const V xw = N::add(N::fma(m1, h, t), W);
+                const V E = N::fma(N::mul(m1, three), W, xw);
+                const V f = N::mul(t, N::fma(t, N::add(t, N::splat(T(-3))), two));
+                const V fp = N::fma(t, N::fma(three, t, N::splat(T(-6))), two);
+                const V pp = N::fma(f, fp, N::mul(m1, N::fma(N::mul(e2, fp), lap, N::mul(ee, f))));
+                const V s1 = N::fma(cp, pp, N::fma(nf2, f, N::mul(c32, t)));
+                P[i] = N::add(N::fma(nf, f, N::mul(c3, t)), E);
+                Q[i] = N::mul(m1, N::fma(two, P[i], s1));
+                R[i] = N::fma(two, s1, E);
+                U[i] = N::mul(m1, N::add(E, xw));
+                m2[i] = N::add(m2[i], N::fma(m1, W, xw));
+            }
+            nest_row_store4<N, RAG>(a.p + row, a.half, start, cnt, j, P);
+            nest_row_store4<N, RAG>(a.q + row, a.half, start, cnt, j, Q);
+            nest_row_store4<N, RAG>(a.r + row, a.half, start, cnt, j, R);
+            nest_row_store4<N, RAG>(a.u + row, a.half, start, cnt, j, U);
+            nest_row_store4<N, RAG>(a.z + row, a.half, start, cnt, j, m2);
+        }
+    }
+    nest_reduce<T>(red, a.red);
+}
+
 }  // namespace molt
