@@ -19,8 +19,8 @@
 //   p = A + E,  q = -(2A + B) - 2p,  r = 2 (2A + B) + E,  u = -E - X W,
 //   W_new = M^{-2} v^n + X W + H_y (u + H_y p) + H_x [ u + H_y (2p - u + H_y q) + H_x (p + H_y (q + H_y r)) ]:
 // one y pass of three fields through two inverses each (NEST_FCH2), one x pass (NEST_ROW_PASS), H_y W_new, and one x pass for
-// v, X W and the next iteration's fields (nest_fch2_kernel): four launches and 100 bytes a point (FP32), the loop on the device: 2048^2, M = 6, 210 us
-// an iteration against 455 by the sweeps, 256^2 30 against 265, FP64 256^2 133 against 520.
+// v, X W and the next iteration's fields (nest_fch2_kernel): four launches and 100 bytes a point (FP32), the loop on
+// the device.  Ten iterations, M = 6, against the sweeps: 2048^2 2.3 / 4.7 ms, 256^2 0.46 / 2.7 ms, FP64 256^2 1.6 / 5.9 ms.
 // Grids with walls or lines that those passes do not take run
 // 14 one-field line sweeps per iteration (11 here, 3 for v, Lap v and X W of the new W; rows
 // through the row kernels, columns through the column kernels), one pointwise kernel and 11 linear

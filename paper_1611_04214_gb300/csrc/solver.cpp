@@ -461,9 +461,9 @@ struct Solver final : molt_solver {
 
     // out = M_{c_out}^{-1} M_{c_in}^{-1} in: one nested pass per axis for equal factors, four sweeps
     // otherwise (scratch f1, f2).
-    cudaError_t rhs_inverse(double c_in, double c_out, const T* in, T* out, cudaStream_t st, bool vch = false) {
+    cudaError_t rhs_inverse(double c_in, double c_out, const T* in, T* out, cudaStream_t st) {
         cudaError_t e;
-        if (use_nest(c_in, c_out, vch)) {
+        if (use_nest(c_in, c_out)) {
             molt::LineParams<T> lx, ly;
             if (!line_params(c_in, 0, &lx) || !line_params(c_in, 1, &ly)) return cudaErrorInvalidValue;
             molt::NestCols<T> c;
@@ -550,16 +550,17 @@ struct Solver final : molt_solver {
     // against the nested ones, M = 4):
     //   FP64: every size (1024^2 510 / 309, 2048^2 1777 / 1072).
     //   FP32: from 256 nodes a side (shorter lines run the block bodies of the batched path, which the
-    //   single grid matches bit for bit); 1024^2 periodic / Neumann 46 / 25 and 60 / 28, 2048^2 92 / 82 and
-    //   128 / 83, 3000 x 2000 276 / 163.  Columns of more than 2048 nodes are spread over clusters of 8 or 16
-    //   blocks whose exchanges cost what the saved traffic gives: 4096^2 Neumann 318 / 292 but periodic
-    //   282 / 295, 2048 x 8192 276 / 332; so there only the grids that the pipelined kernels of the four
-    //   passes serve badly (walls, unaligned lines) and the vector model (767 / 660) take them, up to 4096.
-    bool use_nest(double c_in, double c_out, bool vch = false) const {
+    //   single grid matches bit for bit); 1024^2 periodic / Neumann 46 / 25 and 60 / 28, 2048^2 92 / 77 and
+    //   128 / 78, 4096^2 282 / 272 and 318 / 273, 5000 x 7001 1675 / 1013 and 1732 / 1015, 512 x 8192 143 / 92.  Columns
+    //   of more than 6144 nodes are spread over clusters of 13 to 16 blocks, few of which fit at a time: where the
+    //   rows suit the pipelined kernel of the four passes (whole warps of 16-node chunks from 1024 nodes), those stay,
+    //   2048 x 8192 272 / 325 and 288 / 326, 8192^2 1035 / 1279 and 1072 / 1282; but 1024 x 6000 133 / 117,
+    //   4096 x 6000 409 / 412 and 425 / 415.  Vector model: 4096^2 767 / 590, 2048 x 8192 680 / 697.
+    bool use_nest(double c_in, double c_out) const {
         if (g.dim != 2 || c_in != c_out) return false;
         if (fp32()) {
-            if (g.nx < 256 || g.ny < 256 || g.ny > 4096) return false;
-            if (g.ny > 2048 && !vch && bc == molt::BC_PERIODIC && g.nx % 512 == 0) return false;
+            if (g.nx < 256 || g.ny < 256) return false;
+            if (g.ny > 6144 && g.nx >= 1024 && g.nx % 512 == 0) return false;
         }
         return molt::nest_rows_ok<T>(g.nx) && molt::nest_cols_ok<T>(g.ny);
     }
@@ -615,7 +616,7 @@ struct Solver final : molt_solver {
         ps->g2 = ps->g1 = T(0);
         ps->beta = static_cast<T>(tau / *c_in);
         ps->vch = true;
-        ps->nest = use_nest(*c_in, *c_out, true);
+        ps->nest = use_nest(*c_in, *c_out);
         ps->vs = static_cast<T>((c1 + c2) / tau);
         return true;
     }
@@ -1250,8 +1251,8 @@ struct Solver final : molt_solver {
         Passes ps;
         double c_in, c_out;
         if (!make_vch_passes(tau, &ps, &c_in, &c_out)) return MOLT_ERR_ARG;
-        if ((e = rhs_inverse(c_in, c_out, r1, Y, st, true)) != cudaSuccess ||
-            (e = rhs_inverse(c_in, c_out, r2, vY2, st, true)) != cudaSuccess)
+        if ((e = rhs_inverse(c_in, c_out, r1, Y, st)) != cudaSuccess ||
+            (e = rhs_inverse(c_in, c_out, r2, vY2, st)) != cudaSuccess)
             return cuda_fail(e, "vector CH rhs inverse");
         int it;
         double res, tu;
@@ -1288,8 +1289,8 @@ struct Solver final : molt_solver {
         Passes ps;
         double c_in, c_out;
         if (!make_vch_passes(tau, &ps, &c_in, &c_out)) return MOLT_ERR_ARG;
-        if ((e = rhs_inverse(c_in, c_out, r, Y, st, true)) != cudaSuccess ||
-            (e = rhs_inverse(c_in, c_out, vr2, vY2, st, true)) != cudaSuccess)
+        if ((e = rhs_inverse(c_in, c_out, r, Y, st)) != cudaSuccess ||
+            (e = rhs_inverse(c_in, c_out, vr2, vY2, st)) != cudaSuccess)
             return cuda_fail(e, "vector stage rhs inverse");
         double res, tu;
         molt_status ms = stage(tau, nullptr, st, iters, &res, &tu, true, &ps);
