@@ -922,10 +922,10 @@ __global__ void max_abs_diff_kernel(const T* __restrict__ a, const T* __restrict
     T mt = T(0);
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
          i += static_cast<long long>(gridDim.x) * blockDim.x)
-        mt = fmax(mt, fabs(a[i] - b[i]));
+        mt = abs_max(mt, fabs(a[i] - b[i]));
     double m = static_cast<double>(mt);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(kFull, m, o));
+    for (int o = 16; o > 0; o >>= 1) m = abs_max(m, __shfl_xor_sync(kFull, m, o));
     __shared__ double s[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) s[warp] = m;
@@ -933,7 +933,7 @@ __global__ void max_abs_diff_kernel(const T* __restrict__ a, const T* __restrict
     if (warp == 0) {
         m = lane < static_cast<int>(blockDim.x >> 5) ? s[lane] : 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(kFull, m, o));
+        for (int o = 16; o > 0; o >>= 1) m = abs_max(m, __shfl_xor_sync(kFull, m, o));
         if (lane == 0) atomicMax(out, static_cast<unsigned long long>(__double_as_longlong(m)));
     }
 }

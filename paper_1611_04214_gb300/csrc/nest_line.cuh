@@ -161,8 +161,8 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
         for (int k = 0; k < K; ++k)
             if (k < cnt) {
                 const T nw = y[k] + out[k];
-                dm = fmax(dm, fabs(nw - w[k]));
-                vm = fmax(vm, fabs(nw));
+                dm = abs_max(dm, fabs(nw - w[k]));
+                vm = abs_max(vm, fabs(nw));
                 w[k] = a.fix && (start + k == 0 || start + k == n - 1) ? a.wall : nw;
             }
         dm = nest_warp_max(dm);
@@ -176,8 +176,8 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
             // as loop_check: tolerance, FP32 floor of 2 ulp of max|w|, stall at the FP32 noise floor, cap
             T d = T(0), v = T(0);
             for (int q = 0; q < g.c.nwarps; ++q) {
-                d = fmax(d, s_max[0][q]);
-                v = fmax(v, s_max[1][q]);
+                d = abs_max(d, s_max[0][q]);
+                v = abs_max(v, s_max[1][q]);
             }
             res = static_cast<double>(d);
             const double ulp = static_cast<double>(v) * 5.9604644775390625e-08;

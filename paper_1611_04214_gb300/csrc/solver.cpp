@@ -250,19 +250,22 @@ struct molt_solver {
 
 namespace {
 
+// The larger of two absolute values, a NaN kept.
+double abs_max(double a, double b) { return std::isnan(a) || a > b ? a : b; }
+
 // Step-size control of Algorithm 1 (Sec. 5), with r = eta / lte_tol and q = N_it / N_maxit.
 // A step is accepted when r <= 1 and q < 1.  The next size is dt times a factor: the LTE proposal
 // theta / sqrt(r), capped at gamma while q < 0.7 and at 1 while q < 1 for an accepted step; a
 // rejected step retries with dt / gamma when the LTE was met (so the iteration hit its cap) or
-// r > 2, and with the LTE proposal for 1 < r <= 2.  The result is clipped to [dt_min, dt_max].
-// Returns whether the step is accepted.
+// r > 2 (or r is NaN: a candidate that overflowed), and with the LTE proposal for 1 < r <= 2.  The
+// result is clipped to [dt_min, dt_max].  Returns whether the step is accepted.
 bool step_size_rule(double eta, int n_it, double dt, const molt_adaptive& a, double* next, int max_iter) {
     const double r = eta / a.lte_tol, q = static_cast<double>(n_it) / max_iter;
     const double proposal = eta == 0.0 ? INFINITY : a.theta / std::sqrt(r);
     const bool accept = r <= 1.0 && q < 1.0;
     double factor;
     if (accept) factor = std::min(proposal, q < 0.7 ? a.gamma : 1.0);
-    else factor = (r <= 1.0 || r > 2.0) ? 1.0 / a.gamma : proposal;
+    else factor = (r <= 1.0 || !(r <= 2.0)) ? 1.0 / a.gamma : proposal;
     *next = std::min(std::max(dt * factor, a.dt_min), a.dt_max);
     return accept;
 }
@@ -924,7 +927,7 @@ struct Solver final : molt_solver {
         if (stage_idx < 4) info->iters[stage_idx] = it;
         info->stages = stage_idx + 1;
         info->total_iters += it;
-        info->residual = std::max(info->residual, res);
+        info->residual = abs_max(info->residual, res);
         info->tol_used = tol_used;
     }
 
@@ -1354,7 +1357,7 @@ struct Solver final : molt_solver {
                     ms != MOLT_ERR_NOT_CONVERGED)
                     return ms;
                 n_it = std::max(n_it, it);
-                diff = std::max(max_diff(vb1, va1, st, &e), e == cudaSuccess ? max_diff(vb2, va2, st, &e) : 0.0);
+                diff = abs_max(max_diff(vb1, va1, st, &e), e == cudaSuccess ? max_diff(vb2, va2, st, &e) : 0.0);
             } else {
                 // one BE step into (va), two half steps into (vb)
                 if ((ms = vch_stage_from(u1, u2, 1.0, nullptr, nullptr, 0.0, dt, va1, va2, st, &it)) != MOLT_OK &&
@@ -1370,7 +1373,7 @@ struct Solver final : molt_solver {
                     ms != MOLT_ERR_NOT_CONVERGED)
                     return ms;
                 n_it = std::max(n_it, it);
-                diff = std::max(max_diff(va1, vb1, st, &e), e == cudaSuccess ? max_diff(va2, vb2, st, &e) : 0.0);
+                diff = abs_max(max_diff(va1, vb1, st, &e), e == cudaSuccess ? max_diff(va2, vb2, st, &e) : 0.0);
             }
             if (e != cudaSuccess) return cuda_fail(e, "vector adaptive estimate");
             const double eta = bdf ? diff : 0.5 * diff;   // the factor 1/2 is Richardson's

@@ -189,6 +189,20 @@ struct RedAcc {
     T vmax;   // max |w_new| (stored variable)
 };
 
+// The larger of two absolute values; a NaN on either side stays (fmax would drop it, and an iterate that has
+// overflowed into NaN throughout would leave a residual of zero).  FP64 by bit patterns: non-negative doubles order
+// like them, NaN above infinity, and the integer units are idle beside this part's FP64 units.  (fabs may leave the
+// sign of a NaN set: it is masked here.)
+__device__ __forceinline__ float abs_max(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ double abs_max(double a, double b) {
+    constexpr long long kAbs = 0x7fffffffffffffffLL;
+    return __longlong_as_double(max(__double_as_longlong(a) & kAbs, __double_as_longlong(b) & kAbs));
+}
+
 template <typename T>
 struct OpBase {
     long long ls, ps;
@@ -329,8 +343,8 @@ struct OpP4 : OpBase<T> {
     __device__ __forceinline__ void put(int line, int pos, const T (&h)[1], const T (&a)[NA], RedAcc<T>& r) const {
         const T nw = (a[1] + a[0] - a[2]) + h[0];
         w[this->at(line, pos)] = nw;
-        r.dmax = fmax(r.dmax, fabs(nw - a[0]));
-        r.vmax = fmax(r.vmax, fabs(nw));
+        r.dmax = abs_max(r.dmax, fabs(nw - a[0]));
+        r.vmax = abs_max(r.vmax, fabs(nw));
     }
 };
 
@@ -398,8 +412,8 @@ struct Op1b : OpBase<T> {
     __device__ __forceinline__ void put(int line, int pos, const T (&h)[1], const T (&a)[NA], RedAcc<T>& r) const {
         const T nw = a[1] + h[0];
         w[this->at(line, pos)] = nw;
-        r.dmax = fmax(r.dmax, fabs(nw - a[0]));
-        r.vmax = fmax(r.vmax, fabs(nw));
+        r.dmax = abs_max(r.dmax, fabs(nw - a[0]));
+        r.vmax = abs_max(r.vmax, fabs(nw));
     }
 };
 
@@ -511,8 +525,8 @@ __device__ __forceinline__ void block_reduce_store(RedAcc<T> r, unsigned long lo
     double a = static_cast<double>(r.dmax), b = static_cast<double>(r.vmax);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        a = fmax(a, __shfl_xor_sync(kFull, a, o));
-        b = fmax(b, __shfl_xor_sync(kFull, b, o));
+        a = abs_max(a, __shfl_xor_sync(kFull, a, o));
+        b = abs_max(b, __shfl_xor_sync(kFull, b, o));
     }
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int nthreads = blockDim.x * blockDim.y;
@@ -528,8 +542,8 @@ __device__ __forceinline__ void block_reduce_store(RedAcc<T> r, unsigned long lo
         b = lane < nw ? s_v[lane] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            a = fmax(a, __shfl_xor_sync(kFull, a, o));
-            b = fmax(b, __shfl_xor_sync(kFull, b, o));
+            a = abs_max(a, __shfl_xor_sync(kFull, a, o));
+            b = abs_max(b, __shfl_xor_sync(kFull, b, o));
         }
         if (lane == 0) {
             atomicMax(&slots[0], static_cast<unsigned long long>(__double_as_longlong(a)));
@@ -615,8 +629,8 @@ struct PipeP4 {
                                              RedAcc<T>& r) const {
         const T nw = (av[1] + av[0] - av[2]) + h[0];
         ov[0] = nw;
-        r.dmax = fmax(r.dmax, fabs(nw - av[0]));
-        r.vmax = fmax(r.vmax, fabs(nw));
+        r.dmax = abs_max(r.dmax, fabs(nw - av[0]));
+        r.vmax = abs_max(r.vmax, fabs(nw));
     }
 };
 
@@ -652,8 +666,8 @@ struct Pipe1b {
                                              RedAcc<T>& r) const {
         const T nw = av[1] + h[0];
         ov[0] = nw;
-        r.dmax = fmax(r.dmax, fabs(nw - av[0]));
-        r.vmax = fmax(r.vmax, fabs(nw));
+        r.dmax = abs_max(r.dmax, fabs(nw - av[0]));
+        r.vmax = abs_max(r.vmax, fabs(nw));
     }
 };
 
