@@ -208,6 +208,9 @@ template <typename T>
 cudaError_t nest_fch2(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_t st, long long* launches);
 template <int M, typename T>
 cudaError_t nest_fch2_m(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_t st);
+// The line parameters as the nested passes and the line loop hold them (nest.cpp).
+template <typename T>
+LineParams<T> nest_line_params(const LineParams<T>& lp);
 // Whether the nested passes take lines of n nodes along rows / columns.
 template <typename T>
 bool nest_rows_ok(int n);

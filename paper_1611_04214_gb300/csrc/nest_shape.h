@@ -13,9 +13,6 @@ struct NestCut {
     int nc, rem;
 };
 
-template <typename T>
-LineParams<T> nest_line_params(const LineParams<T>& lp);
-
 namespace detail {
 
 inline bool nest_cut(int n, int K, NestCut* cut) {

@@ -451,21 +451,40 @@ struct Solver final : molt_solver {
                                 &launches);
     }
 
-    // out = M_c^{-1} in = H_x H_y in (2D) or H_x in (1D); uses f1 as scratch in 2D.
-    cudaError_t mm_inv(double c, const T* in, T* out, cudaStream_t st) {
-        molt::LineParams<T> lx, ly;
-        if (!line_params(c, 0, &lx)) return cudaErrorInvalidValue;
-        if (g.dim == 1) return copy_sweep(0, lx, in, out, st, c);
-        if (!line_params(c, 1, &ly)) return cudaErrorInvalidValue;
-        cudaError_t e = copy_sweep(1, ly, in, f1, st);
-        if (e != cudaSuccess) return e;
-        return copy_sweep(0, lx, f1, out, st, c);
+    // The line parameters of single sweeps that go with a nested iteration (nested): its operator's, whose
+    // weights belong to the rounded decay.  A line inverse of other weights differs from it by the rounding of the
+    // decay, which must cancel within a step (see rhs_inverse).
+    bool sweep_params(double c, int axis, bool nested, molt::LineParams<T>* out) {
+        if (!line_params(c, axis, out)) return false;
+        if (nested) *out = molt::nest_line_params(*out);
+        return true;
     }
 
-    // out = M_{c_out}^{-1} M_{c_in}^{-1} in: one nested pass per axis for equal factors, four sweeps
-    // otherwise (scratch f1, f2).
-    cudaError_t rhs_inverse(double c_in, double c_out, const T* in, T* out, cudaStream_t st) {
+    // out = M_c^{-1} in = H_x H_y in (2D) or H_x in (1D); uses f1 as scratch in 2D.
+    cudaError_t mm_inv(double c, const T* in, T* out, cudaStream_t st, bool nested = false) {
+        molt::LineParams<T> lx, ly;
+        const double ct = nested ? 0.0 : c;   // (the tensor-core rows build their own weights from c)
+        if (!sweep_params(c, 0, nested, &lx)) return cudaErrorInvalidValue;
+        if (g.dim == 1) return copy_sweep(0, lx, in, out, st, ct);
+        if (!sweep_params(c, 1, nested, &ly)) return cudaErrorInvalidValue;
+        cudaError_t e = copy_sweep(1, ly, in, f1, st);
+        if (e != cudaSuccess) return e;
+        return copy_sweep(0, lx, f1, out, st, ct);
+    }
+
+    // out = M_{c_out}^{-1} M_{c_in}^{-1} in, by the inverses that the iteration runs: the rounding of their weights
+    // (of d above all) cancels between Y and the iteration; a Y of other inverses drifts by it every step (FP32 SDC2,
+    // 4096 nodes, constant state: 1.5e-7 a step).  The line loop's own inverses for a single line (line: the stage
+    // runs it), one nested pass per axis for equal factors in 2D, four sweeps otherwise (scratch f1, f2).
+    cudaError_t rhs_inverse(double c_in, double c_out, const T* in, T* out, cudaStream_t st, bool line) {
         cudaError_t e;
+        if (line) {
+            molt::LineParams<T> li, lo;
+            if (!line_params(c_in, 0, &li) || !line_params(c_out, 0, &lo)) return cudaErrorInvalidValue;
+            molt::NestLine<T> a;
+            a.w = w, a.r = in, a.Yout = out;
+            return molt::nest_line<T>(li, lo, a, st, &launches);
+        }
         if (use_nest(c_in, c_out)) {
             molt::LineParams<T> lx, ly;
             if (!line_params(c_in, 0, &lx) || !line_params(c_in, 1, &ly)) return cudaErrorInvalidValue;
@@ -482,18 +501,19 @@ struct Solver final : molt_solver {
 
     // out = E_c in with E = M^{-1} - I + D_x D_y, i.e. 2 H_x H_y - H_x - H_y in 2D and H - I in 1D
     // (the operator through which M^{-1} acts on c Lap, Remark Laplacian); scratch f1, f2, f3.
-    cudaError_t e_op(double c, const T* in, T* out, cudaStream_t st) {
+    cudaError_t e_op(double c, const T* in, T* out, cudaStream_t st, bool nested) {
         molt::LineParams<T> lx, ly;
-        if (!line_params(c, 0, &lx)) return cudaErrorInvalidValue;
+        const double ct = nested ? 0.0 : c;
+        if (!sweep_params(c, 0, nested, &lx)) return cudaErrorInvalidValue;
         cudaError_t e;
         if (g.dim == 1) {
-            if ((e = copy_sweep(0, lx, in, f1, st, c)) != cudaSuccess) return e;
+            if ((e = copy_sweep(0, lx, in, f1, st, ct)) != cudaSuccess) return e;
             return lin(out, f1, 1.0, in, -1.0, nullptr, 0, nullptr, 0, 0, st);
         }
-        if (!line_params(c, 1, &ly)) return cudaErrorInvalidValue;
-        if ((e = copy_sweep(1, ly, in, f1, st)) != cudaSuccess) return e;      // H_y
-        if ((e = copy_sweep(0, lx, f1, f2, st, c)) != cudaSuccess) return e;   // H_x H_y
-        if ((e = copy_sweep(0, lx, in, f3, st, c)) != cudaSuccess) return e;   // H_x
+        if (!sweep_params(c, 1, nested, &ly)) return cudaErrorInvalidValue;
+        if ((e = copy_sweep(1, ly, in, f1, st)) != cudaSuccess) return e;       // H_y
+        if ((e = copy_sweep(0, lx, f1, f2, st, ct)) != cudaSuccess) return e;   // H_x H_y
+        if ((e = copy_sweep(0, lx, in, f3, st, ct)) != cudaSuccess) return e;   // H_x
         return lin(out, f2, 2.0, f3, -1.0, f1, -1.0, nullptr, 0, 0, st);
     }
 
@@ -503,19 +523,20 @@ struct Solver final : molt_solver {
     // first.  f(v-1) = w^3 - w for w = v - 1.  Scratch: f1..f6.
     cudaError_t inverse_of_F(const StageParams& sp, const T* w_in, T* out, cudaStream_t st) {
         cudaError_t e;
+        const bool nested = line_loop() || use_nest(sp.c_in, sp.c_out);
         const T* v_in = w_in;
         if (bc == molt::BC_DIRICHLET) {   // Dirichlet E does not kill constants: form v = w + 1
             if ((e = lin(f5, w_in, 1.0, nullptr, 0, nullptr, 0, nullptr, 0, 1.0, st)) != cudaSuccess) return e;
             v_in = f5;
         }
-        if ((e = e_op(sp.c_in, v_in, f4, st)) != cudaSuccess) return e;        // E_i v
-        if ((e = e_op(sp.c_out, f4, f5, st)) != cudaSuccess) return e;         // E_o E_i v
+        if ((e = e_op(sp.c_in, v_in, f4, st, nested)) != cudaSuccess) return e;        // E_i v
+        if ((e = e_op(sp.c_out, f4, f5, st, nested)) != cudaSuccess) return e;         // E_o E_i v
         const bool shifted = shift() == T(1);
         if ((e = molt::cubic<T>(f6, static_cast<long long>(count()), w_in, shifted ? 0.0 : -3.0,
                                 shifted ? -1.0 : 2.0, st, &launches)) != cudaSuccess)
             return e;                                                           // f(v-1)
-        if ((e = e_op(sp.c_in, f6, f4, st)) != cudaSuccess) return e;         // E_i f
-        if ((e = mm_inv(sp.c_out, f4, f6, st)) != cudaSuccess) return e;      // M_o^{-1} E_i f
+        if ((e = e_op(sp.c_in, f6, f4, st, nested)) != cudaSuccess) return e;         // E_i f
+        if ((e = mm_inv(sp.c_out, f4, f6, st, nested)) != cudaSuccess) return e;      // M_o^{-1} E_i f
         return lin(out, f5, -(p.eps * p.eps) / (sp.c_in * sp.c_out), f6, 1.0 / sp.c_in, nullptr, 0, nullptr, 0, 0,
                    st);
     }
@@ -567,6 +588,9 @@ struct Solver final : molt_solver {
         }
         return molt::nest_rows_ok<T>(g.nx) && molt::nest_cols_ok<T>(g.ny);
     }
+
+    // Whether a stage of the scalar model is a single line that the line loop takes.
+    bool line_loop() const { return g.dim == 1 && molt::nest_line_ok<T>(g.nx); }
 
     // The column pass of one field (or component) and the row pass that completes the iterate.
     cudaError_t nest_columns(const Passes& ps, const T* in0, const T* in1, const T* y, T* A, T* B, T* E, int comp,
@@ -813,13 +837,8 @@ struct Solver final : molt_solver {
         a.w = w, a.g2 = ps.g2, a.g1 = ps.g1, a.beta = ps.beta;
         a.tol = p.tol, a.max_iter = p.max_iter, a.ls = ls;
         if (bc == molt::BC_DIRICHLET) {
-            // Y by the loop's own inverses: their rounding (of d above all) cancels between Y and the iteration
-            if (!y_given) {
-                a.r = rhs, a.Yout = Y;
-                if ((e = molt::nest_line<T>(ps.lix, ps.lox, a, st, &launches)) != cudaSuccess)
-                    return cuda_fail(e, "rhs inverse");
-                a.Yout = nullptr;
-            }
+            if (!y_given && (e = rhs_inverse(sp.c_in, sp.c_out, rhs, Y, st, true)) != cudaSuccess)
+                return cuda_fail(e, "rhs inverse");
             if ((e = add_dirichlet_offset(sp, Y, st)) != cudaSuccess) return cuda_fail(e, "Dirichlet offset");
             a.fix = 1, a.wall = T(-1);
             y_given = true;
@@ -846,11 +865,11 @@ struct Solver final : molt_solver {
         if (given) ps = *given;
         else if (!make_passes(sp, &ps)) return MOLT_ERR_ARG;
         cudaError_t e = cudaSuccess;
-        if (g.dim == 1 && !given && molt::nest_line_ok<T>(g.nx))
+        if (!given && line_loop())
             return line_stage(ps, sp, rhs, y_given, st, iters, res_out, tol_out);
         if (!y_given) {
             // Y = M_o^{-1} M_i^{-1} r
-            if ((e = rhs_inverse(sp.c_in, sp.c_out, rhs, Y, st)) != cudaSuccess) return cuda_fail(e, "rhs inverse");
+            if ((e = rhs_inverse(sp.c_in, sp.c_out, rhs, Y, st, false)) != cudaSuccess) return cuda_fail(e, "rhs inverse");
         }
         if (!given && bc == molt::BC_DIRICHLET && (e = add_dirichlet_offset(sp, Y, st)) != cudaSuccess)
             return cuda_fail(e, "Dirichlet offset");
@@ -983,13 +1002,13 @@ struct Solver final : molt_solver {
             return cuda_fail(e, "sdc state");                                  // v0_{n+1}
         if (start) {
             if ((e = lin(r, wn, 1.0, k0, -0.5 * dt, nullptr, 0, nullptr, 0, 0, st)) != cudaSuccess ||
-                (e = rhs_inverse(sp.c_in, sp.c_out, r, Y, st)) != cudaSuccess ||
+                (e = rhs_inverse(sp.c_in, sp.c_out, r, Y, st, line_loop())) != cudaSuccess ||
                 (e = inverse_of_F(sp, v0n, sdc_F0, st)) != cudaSuccess ||
                 (e = lin(Y, Y, 1.0, sdc_F0, 0.5 * dt, nullptr, 0, nullptr, 0, 0, st)) != cudaSuccess)
                 return cuda_fail(e, "sdc rhs");
         } else {
             if ((e = lin(r, wn, 1.0, k0, -0.5 * dt, sdc_F0, 0.5 * dt, nullptr, 0, 0, st)) != cudaSuccess ||
-                (e = rhs_inverse(sp.c_in, sp.c_out, r, Y, st)) != cudaSuccess)
+                (e = rhs_inverse(sp.c_in, sp.c_out, r, Y, st, line_loop())) != cudaSuccess)
                 return cuda_fail(e, "sdc rhs");
         }
         ms = stage(dt, nullptr, st, &it, &res, &tu, true);                     // level [1]
@@ -1254,8 +1273,8 @@ struct Solver final : molt_solver {
         Passes ps;
         double c_in, c_out;
         if (!make_vch_passes(tau, &ps, &c_in, &c_out)) return MOLT_ERR_ARG;
-        if ((e = rhs_inverse(c_in, c_out, r1, Y, st)) != cudaSuccess ||
-            (e = rhs_inverse(c_in, c_out, r2, vY2, st)) != cudaSuccess)
+        if ((e = rhs_inverse(c_in, c_out, r1, Y, st, false)) != cudaSuccess ||
+            (e = rhs_inverse(c_in, c_out, r2, vY2, st, false)) != cudaSuccess)
             return cuda_fail(e, "vector CH rhs inverse");
         int it;
         double res, tu;
@@ -1292,8 +1311,8 @@ struct Solver final : molt_solver {
         Passes ps;
         double c_in, c_out;
         if (!make_vch_passes(tau, &ps, &c_in, &c_out)) return MOLT_ERR_ARG;
-        if ((e = rhs_inverse(c_in, c_out, r, Y, st)) != cudaSuccess ||
-            (e = rhs_inverse(c_in, c_out, vr2, vY2, st)) != cudaSuccess)
+        if ((e = rhs_inverse(c_in, c_out, r, Y, st, false)) != cudaSuccess ||
+            (e = rhs_inverse(c_in, c_out, vr2, vY2, st, false)) != cudaSuccess)
             return cuda_fail(e, "vector stage rhs inverse");
         double res, tu;
         molt_status ms = stage(tau, nullptr, st, iters, &res, &tu, true, &ps);
