@@ -107,7 +107,7 @@ molt_status molt_set_bc(molt_solver* solver, int bc);
  *   the device; the host reads the loop state back once per stage.  Graphs are built on first
  *   use per stage coefficient and reused while parameters, boundary condition and dt are
  *   unchanged.  If a graph cannot be built, the host-driven loop runs instead (counted by
- *   molt_graph_fallbacks).
+ *   molt_graph_fallbacks).  A single line of 32 to 4096 nodes needs no graph: one kernel runs its loop.
  * MOLT_EXEC_HOST_LOOP: the host launches each iteration and reads the residual back after it
  *   (also used while profiling is enabled). */
 typedef enum { MOLT_EXEC_HOST_LOOP = 0, MOLT_EXEC_GRAPH = 1 } molt_execution;
@@ -560,7 +560,8 @@ molt_status molt_profile_enable(molt_solver* solver, int enable);
  * carry kernel = 16, column final kernel of pass k = 17 + k, with k = 0 plain H_c, 1 pass 1,
  * 2 pass 2, 3 pass 3, 4 pass 4, 5 and 6 the two 1D passes.  Nested passes of the 2D iteration
  * with equal factors (two inverses per axis in one kernel): rows = 7, columns = 24, and 15 / 25 for
- * the inverse of a stage's right side. */
+ * the inverse of a stage's right side.  A single line of 32 to 4096 nodes: an iteration in one kernel = 26
+ * (in place of 5 and 6), the inverse of a stage's right side = 27. */
 #define MOLT_PROFILE_SLOTS 32
 molt_status molt_profile_collect(molt_solver* solver, double* ms, long long* launches);
 

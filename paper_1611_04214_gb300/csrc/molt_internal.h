@@ -159,6 +159,7 @@ cudaError_t sweep(int axis, const LineParams<T>& lp, int kind, const OpArgs<T>& 
 // ---- nested passes (nest.cuh, nest_rows.cuh): two inverses of one c along an axis in one pass ----
 // profile slots: the iteration's passes, the rhs inverse
 constexpr int kProfNestRows = 7, kProfNestCols = 24, kProfNestRowsRhs = 15, kProfNestColsRhs = 25;
+constexpr int kProfLine = 26, kProfLineRhs = 27;   // ... of a single line (nest_line.cuh)
 // What a nested column pass computes (nest.cuh).
 enum NestColMode { NEST_SCALAR = 0, NEST_VCH = 1, NEST_Z3 = 2, NEST_COPY = 3, NEST_Y3 = 4, NEST_FCH2 = 5 };
 enum NestRowMode { NEST_ROW_PASS = 0, NEST_ROW_COPY = 1 };
@@ -268,12 +269,13 @@ struct NestLine {
     double tol = 0;
     int max_iter = 0;
     LoopState* ls = nullptr;
+    unsigned long long* red = nullptr;   // (null: not wanted) the last iteration's max |w_new - w| and max |w_new|
 };
 template <typename T>
 bool nest_line_ok(int n);
 template <typename T>
 cudaError_t nest_line(const LineParams<T>& li, const LineParams<T>& lo, const NestLine<T>& p, cudaStream_t st,
-                      long long* launches);
+                      long long* launches, Prof* prof);
 
 // y[j][i] += sum_k a[k][j] b[k][i] (k < terms <= 4), the sum in FP64, for a [ny][nx] field.
 struct Separable {

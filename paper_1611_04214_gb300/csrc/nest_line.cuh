@@ -24,6 +24,7 @@ struct NestLineArgs : NestRowLayout<T> {
     double tol;
     int max_iter, fp32;
     LoopState* ls;
+    unsigned long long* red;   // the last iteration's maxima (may be null)
     NestPow<T> pwo;   // as pw, for the outer inverse
 };
 
@@ -142,7 +143,7 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
         }
     }
     // state of the stopping rule (thread 0)
-    double best = __longlong_as_double(0x7ff0000000000000LL), res = best, tol_used = 0.0;
+    double best = __longlong_as_double(0x7ff0000000000000LL), res = best, vmax = 0.0, tol_used = 0.0;
     int stall = 0, conv = 0, k_it = 0;
     for (;;) {
         V gl[K];
@@ -180,7 +181,8 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
                 v = abs_max(v, s_max[1][q]);
             }
             res = static_cast<double>(d);
-            const double ulp = static_cast<double>(v) * 5.9604644775390625e-08;
+            vmax = static_cast<double>(v);
+            const double ulp = vmax * 5.9604644775390625e-08;
             tol_used = a.fp32 ? fmax(a.tol, 2.0 * ulp) : a.tol;
             ++k_it;
             bool stop = false;
@@ -213,6 +215,10 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
         s.res = res;
         s.tol_used = tol_used;
         *a.ls = s;
+        if (a.red) {
+            a.red[0] = static_cast<unsigned long long>(__double_as_longlong(res));
+            a.red[1] = static_cast<unsigned long long>(__double_as_longlong(vmax));
+        }
     }
 }
 

@@ -483,7 +483,7 @@ struct Solver final : molt_solver {
             if (!line_params(c_in, 0, &li) || !line_params(c_out, 0, &lo)) return cudaErrorInvalidValue;
             molt::NestLine<T> a;
             a.w = w, a.r = in, a.Yout = out;
-            return molt::nest_line<T>(li, lo, a, st, &launches);
+            return molt::nest_line<T>(li, lo, a, st, &launches, &prof);
         }
         if (use_nest(c_in, c_out)) {
             molt::LineParams<T> lx, ly;
@@ -567,6 +567,7 @@ struct Solver final : molt_solver {
         bool two_d;
         bool vch = false;   // vector CH iteration (both components)
         bool nest = false;  // equal factors: one column and one row pass (see the file comment)
+        bool line = false;  // a single line: an iteration is one launch of the line loop
         T vs = 0;           // vector CH: (c1 + c2)/tau
     };
 
@@ -618,6 +619,7 @@ struct Solver final : molt_solver {
         ps->g1 = ps->s == T(1) ? static_cast<T>(sp.lam - 3.0) : static_cast<T>(sp.lam);
         ps->beta = static_cast<T>(sp.beta);
         ps->nest = use_nest(sp.c_in, sp.c_out);
+        ps->line = line_loop();
         return true;
     }
 
@@ -712,10 +714,23 @@ struct Solver final : molt_solver {
         return molt::set_walls<T>(field, g.nx, g.dim == 2 ? g.ny : 1, value, st, &launches);
     }
 
+    // The line loop's arguments but for the right side and the number of iterations.
+    molt::NestLine<T> line_args(const Passes& ps) {
+        molt::NestLine<T> a;
+        a.w = w, a.g2 = ps.g2, a.g1 = ps.g1, a.beta = ps.beta, a.tol = p.tol, a.ls = ls;
+        if (bc == molt::BC_DIRICHLET) a.fix = 1, a.wall = T(-1);
+        return a;
+    }
+
     // One iteration: 2D passes 1-4 (column, row, column, row) or the two 1D row passes.  The
     // last pass accumulates the residual into `red`.
     cudaError_t launch_iteration(const Passes& ps, cudaStream_t st) {
         if (ps.vch) return launch_vch_iteration(ps, st);
+        if (ps.line) {
+            molt::NestLine<T> a = line_args(ps);
+            a.Y = Y, a.max_iter = 1, a.red = red;
+            return molt::nest_line<T>(ps.lix, ps.lox, a, st, &launches, &prof);
+        }
         cudaError_t e;
         if (ps.nest) {
             if ((e = nest_columns(ps, w, nullptr, Y, f1, f2, f3, 0, st)) != cudaSuccess) return e;
@@ -829,23 +844,21 @@ struct Solver final : molt_solver {
         return &lg;
     }
 
-    // A stage of a single line: one kernel runs the whole loop (both execution modes).
+    // A stage of a single line, driven by the device: one kernel runs the whole loop.
     molt_status line_stage(const Passes& ps, const StageParams& sp, const T* rhs, bool y_given, cudaStream_t st, int* iters,
                            double* res_out, double* tol_out) {
         cudaError_t e;
-        molt::NestLine<T> a;
-        a.w = w, a.g2 = ps.g2, a.g1 = ps.g1, a.beta = ps.beta;
-        a.tol = p.tol, a.max_iter = p.max_iter, a.ls = ls;
+        molt::NestLine<T> a = line_args(ps);
+        a.max_iter = p.max_iter;
         if (bc == molt::BC_DIRICHLET) {
             if (!y_given && (e = rhs_inverse(sp.c_in, sp.c_out, rhs, Y, st, true)) != cudaSuccess)
                 return cuda_fail(e, "rhs inverse");
             if ((e = add_dirichlet_offset(sp, Y, st)) != cudaSuccess) return cuda_fail(e, "Dirichlet offset");
-            a.fix = 1, a.wall = T(-1);
             y_given = true;
         }
         a.Y = y_given ? Y : nullptr;
         a.r = rhs;
-        if ((e = molt::nest_line<T>(ps.lix, ps.lox, a, st, &launches)) != cudaSuccess) return cuda_fail(e, "line stage");
+        if ((e = molt::nest_line<T>(ps.lix, ps.lox, a, st, &launches, &prof)) != cudaSuccess) return cuda_fail(e, "line stage");
         if ((e = cudaMemcpyAsync(ls_host, ls, sizeof(molt::LoopState), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
             return cuda_fail(e, "loop state copy");
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "stream sync");
@@ -865,11 +878,11 @@ struct Solver final : molt_solver {
         if (given) ps = *given;
         else if (!make_passes(sp, &ps)) return MOLT_ERR_ARG;
         cudaError_t e = cudaSuccess;
-        if (!given && line_loop())
+        if (ps.line && exec_mode == MOLT_EXEC_GRAPH && !prof.on)
             return line_stage(ps, sp, rhs, y_given, st, iters, res_out, tol_out);
         if (!y_given) {
             // Y = M_o^{-1} M_i^{-1} r
-            if ((e = rhs_inverse(sp.c_in, sp.c_out, rhs, Y, st, false)) != cudaSuccess) return cuda_fail(e, "rhs inverse");
+            if ((e = rhs_inverse(sp.c_in, sp.c_out, rhs, Y, st, ps.line)) != cudaSuccess) return cuda_fail(e, "rhs inverse");
         }
         if (!given && bc == molt::BC_DIRICHLET && (e = add_dirichlet_offset(sp, Y, st)) != cudaSuccess)
             return cuda_fail(e, "Dirichlet offset");

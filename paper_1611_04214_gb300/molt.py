@@ -37,7 +37,8 @@ EXPORTS = [
 ]
 EXECUTION = {"host_loop": 0, "graph": 1}
 PROFILE_SLOTS = 32
-NESTED_SLOTS = {7: "rows_nested", 15: "rows_nested_rhs", 24: "cols_nested", 25: "cols_nested_rhs"}
+NESTED_SLOTS = {7: "rows_nested", 15: "rows_nested_rhs", 24: "cols_nested", 25: "cols_nested_rhs", 26: "line",
+                27: "line_rhs"}
 PASS_NAMES = ["H", "pass1", "pass2", "pass3", "pass4", "pass1d_a", "pass1d_b", ""]
 
 
