@@ -11,6 +11,7 @@
 
 #include "cols_tma.cuh"
 #include "molt_internal.h"
+#include "per_device.h"
 #include "sweep_kernels.cuh"
 
 namespace molt {
@@ -113,7 +114,8 @@ cudaError_t rows(const LineParams<T>& lp, const Op& op, int nlines, unsigned lon
         const int block = lpb * TL < 32 ? 32 : lpb * TL;
         const size_t smem = static_cast<size_t>(lpb) * NF * pitch * sizeof(T);
         auto kern = rows_kernel<T, M, K, Op>;
-        static int limit = smem_optin(kern);
+        static PerDevice limits;
+        const int limit = limits.get([&] { return smem_optin(kern); });
         if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
         const int grid = (nlines + lpb - 1) / lpb;
         prof_begin(prof, kind, st);
@@ -126,7 +128,8 @@ cudaError_t rows(const LineParams<T>& lp, const Op& op, int nlines, unsigned lon
         if (TL > 1024) return cudaErrorInvalidValue;
         const size_t smem = static_cast<size_t>(NF) * pitch * sizeof(T);
         auto kern = rows_kernel<T, M, K, Op>;
-        static int limit = smem_optin(kern);
+        static PerDevice limits;
+        const int limit = limits.get([&] { return smem_optin(kern); });
         if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
         prof_begin(prof, kind, st);
         kern<<<nlines, TL, smem, st>>>(lp, op, nlines, tl_log2, 1, pitch, red);
@@ -261,7 +264,8 @@ cudaError_t rows_pipe_one(const LineParams<float>& lp, const PackedStencil& pw, 
                           size_t smem, unsigned long long* red, cudaStream_t st, Prof* prof, int kind, int rev) {
     const int TL = lp.n / K;
     auto kern = rows_pipe_kernel<M, P, K>;
-    static int limit = smem_optin(kern);
+    static PerDevice limits;
+    const int limit = limits.get([&] { return smem_optin(kern); });
     if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
@@ -298,7 +302,8 @@ cudaError_t rows_pipe(const LineParams<float>& lp, const P& op, int nlines, unsi
         return rows_pipe_one<M, P, 16>(lp, pw, op, nlines, ld, smem, red, st, prof, kind, order & 1);
     } else {
         auto kern = rows_cluster_kernel<M, P, C>;
-        static int limit = smem_optin(kern);
+        static PerDevice limits;
+        const int limit = limits.get([&] { return smem_optin(kern); });
         if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
@@ -361,7 +366,8 @@ cudaError_t cols_pipe_launch(const LineParams<float>& lp, const P& op, int nline
     constexpr int ROWS = kColR + 2 * (kMaxM / 2);
     const size_t smem = static_cast<size_t>(2) * P::NS * ROWS * 32 * sizeof(float);
     auto kern = cols_pipe_kernel<M, P, kFinal>;
-    static int limit = smem_optin(kern);
+    static PerDevice limits;
+    const int limit = limits.get([&] { return smem_optin(kern); });
     if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
@@ -451,7 +457,8 @@ cudaError_t cols_tma_launch(const LineParams<float>& lp, const ColMaps& maps, co
     constexpr int ROWS = kColR + M;
     const size_t smem = static_cast<size_t>(tma_col_stages(P::NS)) * P::NS * ROWS * 32 * sizeof(float) + 128;
     auto kern = cols_tma_kernel<M, P, kFinal>;
-    static int limit = smem_optin(kern);
+    static PerDevice limits;
+    const int limit = limits.get([&] { return smem_optin(kern); });
     if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);

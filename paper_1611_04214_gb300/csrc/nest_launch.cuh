@@ -68,10 +68,11 @@ cudaError_t nest_cols_run(const LineParams<T>& lp, const NestCols<T>& p, cudaStr
     const size_t smem = static_cast<size_t>(nt) * (F::kPitch * sizeof(typename N::V) + 4 * sizeof(T)) +
                         (static_cast<size_t>(2 * F::kNF * (a.slots + 4)) << a.lcp) * sizeof(typename N::V);
     auto kern = F::kern();
-    static int limit = [&] {
+    static PerDevice limits;
+    const int limit = limits.get([&] {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return -1;
         return smem_optin(kern);
-    }();
+    });
     if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -112,7 +113,8 @@ cudaError_t nest_rows_launch(const LineParams<typename N::T>& lp, Args a, cudaSt
     const int block = WARP ? 128 : a.TL;
     const int per = WARP ? block / a.TL : 1;
     const size_t smem = WARP ? 0 : static_cast<size_t>(2 * M) * a.TL * sizeof(typename N::V);
-    static int limit = smem_optin(F::kern());
+    static PerDevice limits;
+    const int limit = limits.get([&] { return smem_optin(F::kern()); });
     if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
     const NestCoef<typename N::V> w = nest_coef<typename N::V, M>(lp);
     // two blocks a SM (the kernel's launch bounds); short lines are on their way before they are wanted

@@ -24,7 +24,8 @@ cudaError_t line_run(const LineParams<T>& li, const LineParams<T>& lo, const Nes
     a.w = p.w, a.Y = p.Y, a.r = p.r, a.Yout = p.Yout, a.g2 = p.g2, a.g1 = p.g1, a.beta = p.beta, a.fix = p.fix, a.wall = p.wall;
     a.tol = p.tol, a.max_iter = p.max_iter, a.fp32 = sizeof(T) == 4, a.ls = p.ls, a.red = p.red;
     auto kern = nest_line_kernel<N, K, M, RAG>;
-    static int limit = smem_optin(kern);
+    static PerDevice limits;
+    const int limit = limits.get([&] { return smem_optin(kern); });
     const size_t smem = 2 * static_cast<size_t>(li.n) * sizeof(T);
     if (limit < 0 || smem > static_cast<size_t>(limit)) return cudaErrorInvalidValue;
     prof_begin(prof, p.Yout ? kProfLineRhs : kProfLine, st);

@@ -30,6 +30,7 @@
 
 #include "cols_tma.cuh"
 #include "molt_internal.h"
+#include "per_device.h"
 
 namespace molt {
 namespace tc {
@@ -270,9 +271,13 @@ rows_kernel(const float* __restrict__ in, float* __restrict__ out, int n, int nl
 template <int M>
 cudaError_t launch(const LineParams<double>& lp, const unsigned char* packed, const float* in, float* out, int nlines,
                    unsigned* status, cudaStream_t st) {
-    static const cudaError_t optin =
-        cudaFuncSetAttribute(rows_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-    if (optin != cudaSuccess) return optin;
+    static PerDevice optin;
+    cudaError_t e = cudaSuccess;
+    const int ok = optin.get([&] {
+        e = cudaFuncSetAttribute(rows_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        return e == cudaSuccess ? 1 : -1;
+    });
+    if (ok < 0) return e != cudaSuccess ? e : cudaErrorInvalidDevice;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
