@@ -16,6 +16,7 @@
 //   Dirichlet  B_a = -(I_0 - mu I_N)/(1-mu^2), B_b = -(I_N - mu I_0)/(1-mu^2)
 // (the Neumann / Dirichlet systems follow from the slope L^{-1}_x = alpha (I^R - I^L) plus the
 // homogeneous part, the way Sec. 3.2 derives the periodic one).
+#include <cfloat>
 #include <cmath>
 #include <cstring>
 
@@ -171,6 +172,28 @@ LineParams<T> cast_line_params(const LineParams<double>& s) {
     return p;
 }
 
+template <typename T>
+double nest_nu(const LineParams<T>& lp) {
+    const double d = static_cast<double>(lp.d);
+    return sizeof(T) == 4 && d >= FLT_MIN && d < 1.0 ? -std::log(d) : static_cast<double>(lp.nu);
+}
+
+template <typename T>
+LineParams<T> nest_line_params(const LineParams<T>& lp) {
+    const double d = static_cast<double>(lp.d);
+    LineParams<double> p;
+    const char* err = nullptr;
+    if (sizeof(T) == 8 || !(d >= FLT_MIN && d < 1.0) || !build_line_params(1.0, nest_nu(lp), lp.n, lp.M, lp.bc, &p, &err))
+        return lp;
+    LineParams<T> q = cast_line_params<T>(p);
+    q.d = lp.d;
+    return q;
+}
+
+template double nest_nu<float>(const LineParams<float>&);
+template double nest_nu<double>(const LineParams<double>&);
+template LineParams<float> nest_line_params<float>(const LineParams<float>&);
+template LineParams<double> nest_line_params<double>(const LineParams<double>&);
 template LineParams<float> cast_line_params<float>(const LineParams<double>&);
 template LineParams<double> cast_line_params<double>(const LineParams<double>&);
 

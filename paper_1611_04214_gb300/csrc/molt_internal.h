@@ -209,7 +209,12 @@ template <typename T>
 cudaError_t nest_fch2(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_t st, long long* launches);
 template <int M, typename T>
 cudaError_t nest_fch2_m(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_t st);
-// The line parameters as the nested passes and the line loop hold them (nest.cpp).
+// The nu of the nested passes and the line loop, nu' = -ln d for the decay d as FP32 kernels hold it, and the line
+// parameters that go with it: recurrence, weights and boundary coefficients then belong to one operator (H 1 = 1 holds
+// with a rounded d too).  They depend on nu alone.  A subnormal d (nu above 87) has few digits left, and -ln d would be
+// up to 3e-3 off nu; H 1 does not feel such a d, and nu stays.
+template <typename T>
+double nest_nu(const LineParams<T>& lp);
 template <typename T>
 LineParams<T> nest_line_params(const LineParams<T>& lp);
 // Whether the nested passes take lines of n nodes along rows / columns.

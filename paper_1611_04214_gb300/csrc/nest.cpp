@@ -1,23 +1,7 @@
 // Entry of the nested passes: eligibility and the dispatch on the quadrature order.
-#include <cmath>
-
 #include "nest_shape.h"
 
 namespace molt {
-
-// The line parameters of nu' = -ln d for the decay d as the kernels hold it: recurrence, weights and boundary
-// coefficients then belong to one operator (H 1 = 1 holds with a rounded d too).  They depend on nu alone.
-template <typename T>
-LineParams<T> nest_line_params(const LineParams<T>& lp) {
-    const double d = static_cast<double>(lp.d);
-    LineParams<double> p;
-    const char* err = nullptr;
-    if (sizeof(T) == 8 || !(d > 0.0 && d < 1.0) || !build_line_params(1.0, -std::log(d), lp.n, lp.M, lp.bc, &p, &err))
-        return lp;
-    LineParams<T> q = cast_line_params<T>(p);
-    q.d = lp.d;
-    return q;
-}
 
 template <typename T>
 bool nest_rows_ok(int n) {
@@ -84,7 +68,6 @@ cudaError_t nest_fch2(const LineParams<T>& lp, const NestFch2<T>& p, cudaStream_
 }
 
 #define MOLT_NEST_ENTRY(T)                                                                                            \
-    template LineParams<T> nest_line_params<T>(const LineParams<T>&);                                                \
     template bool nest_rows_ok<T>(int);                                                                              \
     template bool nest_cols_ok<T>(int);                                                                              \
     template cudaError_t nest_cols<T>(const LineParams<T>&, int, const NestCols<T>&, cudaStream_t, long long*, Prof*); \

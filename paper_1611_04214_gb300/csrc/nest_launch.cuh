@@ -31,7 +31,7 @@ NestCoef<V> nest_coef(const LineParams<T>& lp) {
     NestCoef<V> c;
     std::memset(&c, 0, sizeof(c));
     const double d = static_cast<double>(lp.d);
-    const double nu = sizeof(T) == 4 && d > 0.0 && d < 1.0 ? -std::log(d) : static_cast<double>(lp.nu);
+    const double nu = nest_nu(lp);
     int offs[M + 1];
     double w[M + 1], beta[M + 1];
     for (int o = 0; o <= M; ++o) offs[o] = o - M / 2;
