@@ -181,14 +181,29 @@ struct NestRows {
     T wall = 0;
     unsigned long long* red = nullptr;
 };
+// Constants of a sixth-order step (fch1d.cpp), and as the kernels hold them: the sums are formed in FP64 and rounded
+// once, as the linear combinations of the separate sweeps take them.
+struct FchConsts {
+    double eps2 = 0, eta_eps2 = 0, c_eta = 0, c_f = 0, c_p = 0, inv_a = 0;
+};
+template <typename T>
+struct FchCoef {
+    T eps2, eta_eps2, c_eta, c_f, c_p, inv_a;
+    T c3, c32;   // 3 + c_eta, 3 + 2 c_eta
+};
+template <typename T>
+FchCoef<T> fch_coef(const FchConsts& c) {
+    return {static_cast<T>(c.eps2), static_cast<T>(c.eta_eps2), static_cast<T>(c.c_eta), static_cast<T>(c.c_f),
+            static_cast<T>(c.c_p),  static_cast<T>(c.inv_a),    static_cast<T>(3.0 + c.c_eta),
+            static_cast<T>(3.0 + 2.0 * c.c_eta)};
+}
 // Sixth-order model on independent lines: one iteration in place on v and Lap v (nest_rows.cuh), max |v_new - v|
 // and max |v_new| into red.
 template <typename T>
-struct NestFch {
+struct NestFch : FchConsts {
     T *v = nullptr, *lap = nullptr;
     const T* h2 = nullptr;     // H^2 v^n
     int nlines = 0;
-    double eps2 = 0, eta_eps2 = 0, c_eta = 0, c_f = 0, c_p = 0, inv_a = 0;
     unsigned long long* red = nullptr;
 };
 template <typename T>
@@ -198,11 +213,10 @@ cudaError_t nest_fch_m(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_
 // Sixth-order model in 2D: the x pass that opens an iteration (nest_rows.cuh): v from W and hy = H_y W, the fields
 // p, q, r, u, z of the y pass (NEST_FCH2: in0 .. in2 = p, q, r, U = u, Y = z), max |v_new - v| and max |v_new| into red.
 template <typename T>
-struct NestFch2 {
+struct NestFch2 : FchConsts {
     const T *W = nullptr, *hy = nullptr, *m2 = nullptr;
     T *v = nullptr, *p = nullptr, *q = nullptr, *r = nullptr, *u = nullptr, *z = nullptr;
     int nlines = 0;
-    double eps2 = 0, eta_eps2 = 0, c_eta = 0, c_f = 0, c_p = 0, inv_a = 0;
     unsigned long long* red = nullptr;
 };
 template <typename T>

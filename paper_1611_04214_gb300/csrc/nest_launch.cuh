@@ -223,8 +223,7 @@ cudaError_t nest_fch_m(const LineParams<T>& lp, const NestFch<T>& p, cudaStream_
     using namespace detail;
     NestFchArgs<T> a{};
     a.v = p.v, a.lap = p.lap, a.h2 = p.h2, a.red = p.red;
-    a.eps2 = static_cast<T>(p.eps2), a.eta_eps2 = static_cast<T>(p.eta_eps2), a.c_eta = static_cast<T>(p.c_eta);
-    a.c_f = static_cast<T>(p.c_f), a.c_p = static_cast<T>(p.c_p), a.inv_a = static_cast<T>(p.inv_a);
+    static_cast<FchCoef<T>&>(a) = fch_coef<T>(p);
     const bool al = aligned16(p.v) && aligned16(p.lap) && aligned16(p.h2);
     return nest_rows_run<T, M, NestFchPass>(lp, a, p.nlines, al, st, nullptr, 0);
 }
@@ -234,8 +233,7 @@ cudaError_t nest_fch2_m(const LineParams<T>& lp, const NestFch2<T>& p, cudaStrea
     using namespace detail;
     NestFch2Args<T> a{};
     a.W = p.W, a.hy = p.hy, a.m2 = p.m2, a.v = p.v, a.p = p.p, a.q = p.q, a.r = p.r, a.u = p.u, a.z = p.z, a.red = p.red;
-    a.eps2 = static_cast<T>(p.eps2), a.eta_eps2 = static_cast<T>(p.eta_eps2), a.c_eta = static_cast<T>(p.c_eta);
-    a.c_f = static_cast<T>(p.c_f), a.c_p = static_cast<T>(p.c_p), a.inv_a = static_cast<T>(p.inv_a);
+    static_cast<FchCoef<T>&>(a) = fch_coef<T>(p);
     bool al = true;
     const T* fields[] = {p.W, p.hy, p.m2, p.v, p.p, p.q, p.r, p.u, p.z};
     for (const T* f : fields) al = al && aligned16(f);

@@ -465,11 +465,10 @@ nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
 // 1024 nodes, FP32, M = 6: 107 us an iteration = 3100 GB/s of the 20 B a point, fourteen kernels took 606; FP64, 4096
 // lines: 670 us, FP64 units, against 1856.
 template <typename T>
-struct NestFchArgs : NestRowLayout<T> {
+struct NestFchArgs : NestRowLayout<T>, FchCoef<T> {
     T* v;
     T* lap;
     const T* h2;
-    T eps2, eta_eps2, c_eta, c_f, c_p, inv_a;
     unsigned long long* red;
 };
 
@@ -487,7 +486,7 @@ nest_fch_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     NestRowThread<N> g = nest_row_thread<N, K, RAG, WARP>(lp, a);
     const int start = g.start, cnt = g.ck.cnt;
     const size_t row = g.row;
-    const V m1 = N::splat(T(-1)), c3 = N::splat(T(3) + a.c_eta), nf = N::splat(-a.c_f);
+    const V m1 = N::splat(T(-1)), c3 = N::splat(a.c3), nf = N::splat(-a.c_f);
     auto cube = [&](V x) { return N::mul(x, N::fma(x, N::add(x, N::splat(T(-3))), N::splat(T(2)))); };   // f(v)
 
     V x[K + M], out[K];
@@ -580,10 +579,9 @@ __device__ __forceinline__ void nest_row_store4(typename N::T* f, int half, int 
 // Bound: latency of two line chains at 16 warps a SM and 40 B a point: 2048^2 FP32, M = 6: 60 us = 2800 GB/s.  The whole
 // iteration (y pass 97, x pass 28, H_y W 22, this 60 us) takes 210 us; fourteen sweeps and twelve other kernels took 455.
 template <typename T>
-struct NestFch2Args : NestRowLayout<T> {
+struct NestFch2Args : NestRowLayout<T>, FchCoef<T> {
     const T *W, *hy, *m2;
     T *v, *p, *q, *r, *u, *z;
-    T eps2, eta_eps2, c_eta, c_f, c_p, inv_a;
     unsigned long long* red;
 };
 
@@ -629,7 +627,7 @@ nest_fch2_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     nest_row_inverse<N, K, M, RAG, WARP>(lp, w, a, g, sh, edge + 2 * H * a.TL, x, out);
     if (g.on) {
         const V e2 = N::splat(a.eps2), ee = N::splat(a.eta_eps2), cp = N::splat(a.c_p), nf = N::splat(-a.c_f);
-        const V c3 = N::splat(T(3) + a.c_eta), c32 = N::splat(T(3) + T(2) * a.c_eta), nf2 = N::splat(T(-2) * a.c_f);
+        const V c3 = N::splat(a.c3), c32 = N::splat(a.c32), nf2 = N::splat(T(-2) * a.c_f);
         const V ia = N::splat(a.inv_a);
 #pragma unroll
         for (int j = 0; j < K / 4; ++j) {
