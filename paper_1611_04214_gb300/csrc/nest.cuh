@@ -103,6 +103,17 @@ __device__ __forceinline__ void nest_ghosts(const NestChunk& c, typename N::V (&
     }
 }
 
+// R_k + sum_m gamma_m x[k+m]; Q_k is added last, so that the sum rounds at the size of one half of the output (Q and R
+// are about half of it each) and not of all of it.
+template <class N, int M, int KM>
+__device__ __forceinline__ typename N::V nest_stencil(const NestCoef<typename N::V>& w, const typename N::V (&x)[KM], int k,
+                                                      typename N::V r) {
+    constexpr int H = M / 2;
+#pragma unroll
+    for (int m = 0; m < H; ++m) r = N::fma(w.gamma[m], N::add(x[k + m], x[k + M - m]), r);
+    return N::fma(w.gamma[H], x[k + H], r);
+}
+
 // Zero-start aggregates of a chunk of CNT nodes: P^L at its last node and P^R at its first one with
 // nothing entering (I^L_0 = 0 and I^R_N = 0 at walls).  pw = d^(CNT-1).
 template <class N, int M, int CNT, int KM>
@@ -117,17 +128,18 @@ __device__ __forceinline__ void nest_agg(const NestCoef<typename N::V>& w, typen
         s = N::fma(dv, s, x[k]);
         r = N::fma(dv, r, x[CNT - 1 - k + M]);
     }
-    V a = N::mul(w.alpha, s), b = N::mul(w.alpha, r);
+    // (the large term last: the sums before it round at the size of the weights)
+    V a = N::mul(w.beta[1], x[CNT]), b = N::mul(w.beta[1], x[M - 1]);
     V ka = N::mul(w.beta[1], x[0]), kb = N::mul(w.beta[1], x[CNT - 1 + M]);
 #pragma unroll
-    for (int i = 1; i <= M; ++i) {
+    for (int i = 2; i <= M; ++i) {
         a = N::fma(w.beta[i], x[CNT - 1 + i], a);
         b = N::fma(w.beta[i], x[M - i], b);
-        if (i > 1) {
-            ka = N::fma(w.beta[i], x[i - 1], ka);
-            kb = N::fma(w.beta[i], x[CNT - i + M], kb);
-        }
+        ka = N::fma(w.beta[i], x[i - 1], ka);
+        kb = N::fma(w.beta[i], x[CNT - i + M], kb);
     }
+    a = N::fma(w.alpha, s, a);
+    b = N::fma(w.alpha, r, b);
     ka = N::mul(nd, ka);
     kb = N::mul(nd, kb);
     if (c.mA | c.mB) {
@@ -180,10 +192,7 @@ __device__ __forceinline__ void nest_finish(const NestCoef<typename N::V>& w, ty
 #pragma unroll
     for (int k = 0; k < CNT; ++k) {
         if (k > 0) q = N::fma(dv, q, N::mul(w.alpha, x[k]));
-        V e = N::fma(w.gamma[H], x[k + H], N::add(out[k], q));
-#pragma unroll
-        for (int m = 0; m < H; ++m) e = N::fma(w.gamma[m], N::add(x[k + m], x[k + M - m]), e);
-        out[k] = e;
+        out[k] = N::add(nest_stencil<N, M>(w, x, k, out[k]), q);
     }
 }
 
@@ -238,17 +247,18 @@ __device__ __forceinline__ void nest_agg_wall(const LineParams<typename N::T>& l
         s = N::fma(dv, s, x[k]);
         r = N::fma(dv, r, x[CNT - 1 - k + M]);
     }
-    V a = N::mul(w.alpha, s), b = N::mul(w.alpha, r);
+    // (the large term last: the sums before it round at the size of the weights)
+    V a = N::mul(w.beta[1], x[CNT]), b = N::mul(w.beta[1], x[M - 1]);
     V ka = N::mul(w.beta[1], x[0]), kb = N::mul(w.beta[1], x[CNT - 1 + M]);
 #pragma unroll
-    for (int i = 1; i <= M; ++i) {
+    for (int i = 2; i <= M; ++i) {
         a = N::fma(w.beta[i], x[CNT - 1 + i], a);
         b = N::fma(w.beta[i], x[M - i], b);
-        if (i > 1) {
-            ka = N::fma(w.beta[i], x[i - 1], ka);
-            kb = N::fma(w.beta[i], x[CNT - i + M], kb);
-        }
+        ka = N::fma(w.beta[i], x[i - 1], ka);
+        kb = N::fma(w.beta[i], x[CNT - i + M], kb);
     }
+    a = N::fma(w.alpha, s, a);
+    b = N::fma(w.alpha, r, b);
     aL = N::fma(pv, N::mul(nd, ka), a);
     aR = N::fma(pv, N::mul(nd, kb), b);
     if (c.mA | c.mB) {
@@ -352,10 +362,7 @@ __device__ __forceinline__ void nest_finish_wall(const LineParams<typename N::T>
         if (k > 0) q = N::fma(dv, q, N::mul(w.alpha, x[k]));
         if (k == H - 1 && c.mA) q = N::blend(q, qs, c.mA);
         if (k == CNT - 1 - H) ql = q;
-        V e = N::fma(w.gamma[H], x[k + H], N::add(out[k], q));
-#pragma unroll
-        for (int m = 0; m < H; ++m) e = N::fma(w.gamma[m], N::add(x[k + m], x[k + M - m]), e);
-        out[k] = e;
+        out[k] = N::add(nest_stencil<N, M>(w, x, k, out[k]), q);
     }
     if (c.mA) {
 #pragma unroll
