@@ -40,13 +40,25 @@ METRIC = "Helmholtz line-sweep Gpts/s (% HBM peak); CH steps/s vs FP64 path at â
 UNIT = "Gpts/s"
 WORKLOAD = dict(name="ch2d_8192_sdirk3_periodic", n=8192, eps=0.02, dt=5e-5, scheme="sdirk3", bc="periodic",
                 M=4, mean=0.1, amp=0.05, seed=0, L=6.283185307179586)
-SWEEPS_RHS, SWEEPS_ITER = 4, 7          # field sweeps per stage rhs inverse / per 2D iteration
+SWEEPS_RHS, SWEEPS_ITER = 4, 7          # field sweeps per stage rhs inverse / per 2D iteration (four passes)
 # (fields read, fields written) per point, algorithmic (each needed value moved once)
 KERNEL_FIELDS = {
     "rows_H": (1, 1), "rows_pass2": (3, 2), "rows_pass4": (5, 1),
     "cols_agg_H": (1, 0), "cols_agg_pass1": (1, 0), "cols_agg_pass3": (2, 0),
     "cols_final_H": (1, 1), "cols_final_pass1": (1, 2), "cols_final_pass3": (2, 2),
+    "cols_nested": (2, 3), "rows_nested": (4, 1), "cols_nested_rhs": (1, 1), "rows_nested_rhs": (1, 1),
 }
+
+
+def path_counts(kernels):
+    """(field sweeps of a stage's rhs inverse, of a 2D iteration; words per point of each) by the kernels that ran: nested
+    passes (four inverses of the column pass, two of the row pass) or the four fused passes."""
+    if "cols_nested" in kernels:
+        words = [sum(sum(KERNEL_FIELDS[f"{a}_nested{b}"]) for a in ("cols", "rows")) for b in ("_rhs", "")]
+        return SWEEPS_RHS, 6, words[0], words[1]
+    return SWEEPS_RHS, SWEEPS_ITER, SWEEPS_RHS * 2, 18
+
+
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) measured by ncu for the
 # kernels of the workloads, keyed by kernel slot, with the pass and kernel family captured; filled
 # only for kernels unchanged since their capture, and reported only when the autotuner kept the
@@ -409,7 +421,7 @@ VCH = dict(VCH_WORKLOADS["mixture"])
 # field words moved per point by one vector CH iteration (two components): the nested column and row
 # pass of each component read / write 3+3 and 4+1 fields; each stage's rhs inverses 2 x (1+1) per component
 VCH_WORDS_ITER, VCH_WORDS_RHS = 22, 8
-VCH_SWEEPS_ITER, VCH_SWEEPS_RHS = 14, 8
+VCH_SWEEPS_ITER, VCH_SWEEPS_RHS = 12, 8
 # (read, write) fields per point of each vector CH kernel slot; the vector passes 1 and 2 read
 # both components (the column aggregate of pass 1 reads them once more)
 VCH_KERNEL_FIELDS = {
@@ -632,17 +644,17 @@ CONVERGED_WL = dict(name="ch2d_1024_neumann_bdf2_converged", n=1024, eps=0.05, d
 
 SPLIT3D = dict(name="ch3d_256_be_periodic", n=256, eps=0.05, dt=1e-4, M=4, amp=0.05, seed=0, iters=10, steps=3)
 # per 3D iteration (equal factors): the z pass reads w and writes three fields (16 B/pt), the y pass reads
-# those and Y and writes three (28 B/pt), the x pass reads three fields and w and writes w (20 B/pt), two line
-# inverses of two or three fields each (15 of the separate form); the rhs inverse's three copies 8 B/pt each
+# those and Y and writes three (28 B/pt), the x pass reads three fields and w and writes w (20 B/pt); two line
+# inverses of two, three and one field (15 sweeps in the separate form); the rhs inverse's three copies 8 B/pt each
 SPLIT3D_BYTES_ITER, SPLIT3D_BYTES_RHS = 16 + 28 + 20, 3 * 8
-SPLIT3D_SWEEPS_ITER, SPLIT3D_SWEEPS_RHS = 15, 6
+SPLIT3D_SWEEPS_ITER, SPLIT3D_SWEEPS_RHS = 4 + 6 + 2, 6
 
 
 def split3d_leg():
     """The 3D split stage (molt_solver3d_*; the extension of the splitting that Sec. 5 remarks on)
     on a 256^3 periodic grid over [0, 2pi]^3: eps = 0.05, BE dt = 1e-4, u0 = 0.05 U[-1, 1]
     (SplitMix64, seed 0), a fixed 10 fixed-point iterations per stage.  Line-sweep points per second
-    and the step's algorithmic HBM fraction; the passes are not fused."""
+    and the step's algorithmic HBM fraction (one nested pass per axis)."""
     import torch
 
     from paper_1611_04214_gb300.inputs import uniform_noise
@@ -691,7 +703,7 @@ def fch1d_leg():
     there; at the paper's dt = 0.1 it does not), each line the 1D initial state of Eq. CH1D_initial
     plus 0.05 U[-1, 1] (SplitMix64, seed 0), a fixed 20 iterations per step, FP32 and FP64.  Every
     field (67 MB FP32) is larger than L2.  Line-sweep points per second and the algorithmic HBM
-    fraction of the step (the iteration's kernels are not fused)."""
+    fraction of the step (an iteration is one kernel)."""
     import torch
 
     from paper_1611_04214_gb300.inputs import paper_ic_1d, uniform_noise
@@ -749,7 +761,7 @@ def fch2d_leg():
     as in Sec. 5.1) of 4096^2 over [0, 2pi]^2: eps = 0.18, eta = 1, BE dt = 0.05, the 2D initial
     state of Eq. CH2D_initial plus 0.05 U[-1, 1] (SplitMix64, seed 0), a fixed 10 iterations per
     step, FP32 and FP64.  Every FP32 field (67 MB) is larger than L2.  Line-sweep points per
-    second and the algorithmic HBM fraction of the step (the regrouped, unfused iteration)."""
+    second and the algorithmic HBM fraction of the step (four kernels an iteration)."""
     import torch
 
     from paper_1611_04214_gb300.inputs import paper_ic_2d, uniform_noise
@@ -942,11 +954,9 @@ def run_ours(args, rank, world, dist):
     clocks.start()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     ev0.record(stream)
-    sweeps, infos = 0, []
+    infos = []
     for _ in range(args.steps):
-        info = step()
-        infos.append(info)
-        sweeps += sum(SWEEPS_RHS + SWEEPS_ITER * k for k in info.iters)
+        infos.append(step())
     ev1.record(stream)
     torch.cuda.synchronize()
     clocks.stop()
@@ -956,6 +966,8 @@ def run_ours(args, rank, world, dist):
     ms = ev0.elapsed_time(ev1)
     prof = solver.profile_collect()
     solver.profile_enable(False)
+    sweeps_rhs, sweeps_iter, words_rhs, words_iter = path_counts(prof)
+    sweeps = sum(sweeps_rhs + sweeps_iter * k for i in infos for k in i.iters)
     ms, pts_total = combine_ranks(ms, sweeps * n * n, dist)
     value = pts_total / (ms * 1e-3) / 1e9
 
@@ -976,10 +988,10 @@ def run_ours(args, rank, world, dist):
     kernels = {k: {"ms_total": v[0], "launches": v[1], "gbs": (
         (KERNEL_FIELDS[k][0] + KERNEL_FIELDS[k][1]) * elem * n * n / (v[0] / v[1] * 1e-3) / 1e9
         if k in KERNEL_FIELDS else None)} for k, v in prof.items()}
-    # whole-step algorithmic HBM fraction: per iteration 72 B/pt (FP32), per rhs inverse 4 sweeps x 8 B/pt
+    # whole-step algorithmic HBM fraction: four passes 72 B/pt an iteration (FP32) and 4 sweeps x 8 B/pt an rhs inverse
     iters_total = sum(sum(i.iters) for i in infos)
     stages_total = sum(len(i.iters) for i in infos)
-    step_bytes = (iters_total * 18 + stages_total * 4 * 2) * elem * n * n
+    step_bytes = (iters_total * words_iter + stages_total * words_rhs) * elem * n * n
     hbm_frac_step = step_bytes / (ms * 1e-3) / 1e9 / peak
 
     result = None
@@ -990,7 +1002,7 @@ def run_ours(args, rank, world, dist):
         e2e_pts, t0 = 0, time.perf_counter()
         for _ in range(e2e_steps):
             info = solver.run_host(uh, WORKLOAD["dt"], WORKLOAD["scheme"], 1, raise_on_nonconvergence=False)
-            e2e_pts += sum(SWEEPS_RHS + SWEEPS_ITER * k for k in info.iters) * n * n
+            e2e_pts += sum(sweeps_rhs + sweeps_iter * k for k in info.iters) * n * n
         e2e_secs = time.perf_counter() - t0
         e2e = {"value": e2e_pts / e2e_secs / 1e9, "unit": UNIT, "h2d_bytes_per_step": n * n * elem,
                "d2h_bytes_per_step": n * n * elem, "steps": e2e_steps}
