@@ -15,7 +15,11 @@ value = line-sweep points per second (Gpts/s) over the whole step: sum of field 
 points / device time.  Every field is 256 MiB, larger than the 129 MB L2, so no flush is
 needed between steps.
 
-Side legs on the same JSON line:
+One JSON line on stdout holds the main workload and one figure of every side leg, short enough to be
+kept whole by a reader that records the end of the output (``headline``).  Everything measured, one
+JSON line too, goes to stderr.
+
+Side legs:
 - the FP64 GPU path on the same start;
 - 512 batched instances;
 - single sweeps;
@@ -254,6 +258,50 @@ def run_reference(args, rank):
             "cpu_baseline": {"value": value, "unit": UNIT, "cores": procs, "kind": "oracle", "sample": sample},
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
     print(json.dumps(line), flush=True)
+
+
+# keys of the full record that the line on stdout keeps, in order
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "roofline", "cpu_baseline", "e2e", "gpu_launches", "clocks",
+            "iters_per_stage", "final_residual", "hbm_frac_step_algorithmic", "ms_per_step_graph_mode", "fp32_vs_fp64",
+            "ch2d8192_crop1024_err_vs_oracle")
+HEADLINE_BYTES = 2800
+# one figure of every side leg: (name on the line, path in the full record)
+LEG_FIGURES = (("batched_ms", ("batched", "ms_per_step")),
+               ("converged_steps_per_s", ("converged_l2_resident", "fp32", "steps_per_s")),
+               ("vector_ch_ms", ("vector_ch", "fp32", "ms_per_step")), ("split3d_ms", ("split3d", "ms_per_step")),
+               ("fch1d_ms", ("fch1d", "fp32", "ms_per_step")), ("fch2d_ms", ("fch2d", "fp32", "ms_per_step")))
+
+
+def _rounded(x):
+    """Floats to six significant digits, throughout."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: _rounded(v) for k, v in x.items()}
+    return [_rounded(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def headline(res) -> str:
+    """The line on stdout: the main workload and a figure of every side leg, at most HEADLINE_BYTES long (what the
+    record's texts take beyond that is cut from the samples' descriptions)."""
+    line = {k: res[k] for k in HEADLINE if k in res}
+    legs = {}
+    for name, path in LEG_FIGURES:
+        v = res
+        for k in path:
+            v = v.get(k) if isinstance(v, dict) else None
+        if v is not None:
+            legs[name] = v
+    if legs:
+        line["legs"] = legs
+    line = _rounded(line)
+    for key, text in (("cpu_baseline", "sample"), ("roofline", "traffic_last_capture"), ("config", "initial_state")):
+        if len(json.dumps(line)) <= HEADLINE_BYTES:
+            break
+        if isinstance(line.get(key), dict) and text in line[key]:
+            line[key] = {**line[key], text: str(line[key][text])[:60]}
+    return json.dumps(line)
 
 
 def _config(args):
@@ -1159,7 +1207,8 @@ def main():
         dist.barrier()
     res = run_ours(args, rank, world, dist)
     if rank == 0 and res is not None:
-        print(json.dumps(res), flush=True)
+        print(json.dumps(_rounded(res)), file=sys.stderr, flush=True)
+        print(headline(res), flush=True)
     if dist:
         dist.destroy_process_group()
 
