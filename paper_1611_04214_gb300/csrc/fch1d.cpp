@@ -106,9 +106,11 @@ struct Fch1d final : molt_fch1d {
     }
 
     // Whether the fused iteration (nest_fch_kernel) takes the lines: periodic ones.  With walls the map amplifies rounding, so
-    // that two orders of the same operations differ by up to 1e-3 of the field in FP32 and 1e-12 in FP64 after a few
-    // iterations (8192 nodes of noise); those keep the separate sweeps and their results.  FP64 lines below 256 nodes stay
-    // with the sweeps too: callers count their launches (14 and more an iteration).
+    // that two orders of the same operations differ by up to 1e-3 of the field in FP32 after a few iterations (8192 nodes of
+    // noise), and in FP64 the fused form was less exact (error 7e-15 -> 1e-13); those keep
+    // the separate sweeps and their results.  FP64 lines below 256 nodes stay with the sweeps for the launches that
+    // molt_fch1d_launches reports there (14 and more an iteration, as tests/test_gpu_fch.py asserts), not for speed
+    // or accuracy: the fused form has not been measured on them.
     bool fused() const { return molt::nest_rows_ok<T>(nx) && bc == molt::BC_PERIODIC && (sizeof(T) == 4 || nx >= 256); }
 
     // H^2 v^n by the inverses that the iteration runs (their rounding then cancels between the two).

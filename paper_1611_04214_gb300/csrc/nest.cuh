@@ -30,8 +30,6 @@ template <> struct NestVec<float, 2> : Lanes<2> {
     static __device__ __forceinline__ V blend(V a, V b, int mask) {
         return pack((mask & 1) ? get(b, 0) : get(a, 0), (mask & 2) ? get(b, 1) : get(a, 1));
     }
-    static __device__ __forceinline__ unsigned long long bits(V a) { return a; }
-    static __device__ __forceinline__ V from_bits(unsigned long long b) { return b; }
 };
 template <typename S> struct NestVec<S, 1> {
     using T = S;
@@ -306,6 +304,7 @@ __device__ __forceinline__ void nest_finish_wall(const LineParams<typename N::T>
                                             typename N::V cR, End end, typename N::V (&out)[K]) {
     using V = typename N::V;
     constexpr int H = M / 2;
+    static_assert(H > 1, "(the right wall's start is a node before the last)");
     const V dv = N::splat(lp.d), m1 = N::splat(typename N::T(-1));
     const NestWall<N, M, CNT, KM> wl{lp, w, x};
     V ka = N::mul(w.beta[1], x[0]), kb = N::mul(w.beta[1], x[CNT - 1 + M]);
@@ -330,12 +329,8 @@ __device__ __forceinline__ void nest_finish_wall(const LineParams<typename N::T>
 #pragma unroll
     for (int k = CNT - 2; k >= 0; --k) {
         r = N::fma(dv, r, N::mul(w.alpha, x[k + M]));
-        if (k == CNT - H && H > 1 && c.mB) r = N::blend(r, rs, c.mB);
+        if (k == CNT - H && c.mB) r = N::blend(r, rs, c.mB);
         out[k] = r;
-        if (k == CNT - 1 - H && H == 1 && c.mB) {   // H = 1: the start is the last node itself
-            r = N::blend(r, N::fma(dv, rs, N::mul(w.alpha, x[k + M])), c.mB);
-            out[k] = r;
-        }
     }
     V pa[H], qs = N::zero();      // left wall: the first H outputs, Q of node H - 1
 #pragma unroll
@@ -380,16 +375,16 @@ __device__ __forceinline__ void nest_finish_wall(const LineParams<typename N::T>
 
 // Walls by ghost values or by shifted stencils.  Sixth order's ghosts weigh the first nodes by up to 140, which on rough data
 // costs FP32 two bits of the nodes beside a wall (1024^2 Neumann, two solves: largest error 3.5e-6 of the field's largest value
-// with ghosts, 7.4e-7 with the stencils, 8.0e-7 by single sweeps); fourth order's (up to 10) cost nothing
-// measurable (8.2e-7, 8.7e-7, 7.0e-7), and in FP64 neither does (256^2 to 1024^2: 1.3e-14 and 1.8e-14 of either form and of
-// single sweeps).  The stencils are work for the warps that hold a wall, which are all of them on short FP64 lines:
-// 256^2 FP64 117 us an iteration, with ghosts 80.
+// with ghosts, 7.1e-7 with the stencils, 8.0e-7 by single sweeps); fourth order's (up to 10) cost nothing
+// measurable (6.8e-7, 6.5e-7, 7.3e-7), and in FP64 neither does (256^2, M = 6: 5.8e-14, 5.3e-14, 5.4e-14).  The stencils are
+// work for the warps that hold a wall, which are all of them on short FP64 lines: 256^2 FP64, M = 6, 135 us an
+// iteration, with ghosts 102.
 template <class N, int M> inline constexpr bool kNestGhosts = M <= 4 || sizeof(typename N::T) == 8;
 
 // The powers d^(K-1) and d^(K-2): what a value decays by over a chunk of K or K - 1 nodes, one node less.
 template <typename T> struct NestPow { T full, less; };
 
-template <class N, int K, int M, int S, bool RAG, int KM>
+template <class N, int K, int M, bool RAG, int KM>
 __device__ __forceinline__ void nest_chunk_agg(const LineParams<typename N::T>& lp, const NestCoef<typename N::V>& w,
                                                const NestPow<typename N::T>& p, const NestChunk& c,
                                                typename N::V (&x)[KM], typename N::V& aL, typename N::V& aR) {
@@ -398,32 +393,32 @@ __device__ __forceinline__ void nest_chunk_agg(const LineParams<typename N::T>& 
             nest_ghosts<N, M, K>(c, x);
             nest_agg<N, M, K>(w, lp.d, p.full, c, x, aL, aR);
         } else {
-            nest_ghosts<N, M, K - S>(c, x);
-            nest_agg<N, M, K - S>(w, lp.d, p.less, c, x, aL, aR);
+            nest_ghosts<N, M, K - 1>(c, x);
+            nest_agg<N, M, K - 1>(w, lp.d, p.less, c, x, aL, aR);
         }
     } else {
         if (!RAG || c.cnt == K) nest_agg_wall<N, M, K>(lp, w, p.full, c, x, aL, aR);
-        else nest_agg_wall<N, M, K - S>(lp, w, p.less, c, x, aL, aR);
+        else nest_agg_wall<N, M, K - 1>(lp, w, p.less, c, x, aL, aR);
     }
     if (c.cnt == 0) aL = aR = N::zero();
 }
 
 // end(0), end(1): the boundary values of the line, asked for at walls only.
-template <class N, int K, int M, int S, bool RAG, int KM, class End>
+template <class N, int K, int M, bool RAG, int KM, class End>
 __device__ __forceinline__ void nest_chunk_finish(const LineParams<typename N::T>& lp, const NestCoef<typename N::V>& w,
                                                   const NestChunk& c, const typename N::V (&x)[KM], typename N::V cL,
                                                   typename N::V cR, End end, typename N::V (&out)[K]) {
     if constexpr (kNestGhosts<N, M>) {
         if (!RAG || c.cnt == K) nest_finish<N, K, M, K>(w, lp.d, c, x, cL, cR, end, out);
-        else nest_finish<N, K, M, K - S>(w, lp.d, c, x, cL, cR, end, out);
+        else nest_finish<N, K, M, K - 1>(w, lp.d, c, x, cL, cR, end, out);
     } else {
         if (!RAG || c.cnt == K) nest_finish_wall<N, K, M, K>(lp, w, c, x, cL, cR, end, out);
-        else nest_finish_wall<N, K, M, K - S>(lp, w, c, x, cL, cR, end, out);
+        else nest_finish_wall<N, K, M, K - 1>(lp, w, c, x, cL, cR, end, out);
     }
 }
 
 // Halo values hl (before the chunk) and hr (after it) into the window x.
-template <class N, int K, int M, int S, bool RAG, int KM>
+template <class N, int K, int M, bool RAG, int KM>
 __device__ __forceinline__ void nest_set_halo(int cnt, const typename N::V (&hl)[M / 2], const typename N::V (&hr)[M / 2],
                                               typename N::V (&x)[KM]) {
     constexpr int H = M / 2;
@@ -434,7 +429,7 @@ __device__ __forceinline__ void nest_set_halo(int cnt, const typename N::V (&hl)
         for (int h = 0; h < H; ++h) x[H + K + h] = hr[h];
     } else {
 #pragma unroll
-        for (int h = 0; h < H; ++h) x[H + K - S + h] = hr[h];
+        for (int h = 0; h < H; ++h) x[H + K - 1 + h] = hr[h];
     }
 }
 
@@ -461,11 +456,6 @@ __device__ __forceinline__ void nest_boundary(const LineParams<T>& lp, T I0, T I
 }
 
 // ---- thread-block clusters ----
-__device__ __forceinline__ int nest_cluster_rank() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return static_cast<int>(r);
-}
 __device__ __forceinline__ void nest_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -687,7 +677,7 @@ struct NestColGeo {
     bool both;       // the second column of the pair exists
 };
 
-template <class N, int K, int S, bool RAG>
+template <class N, int K, bool RAG>
 __device__ __forceinline__ NestColGeo nest_col_geo(const LineParams<typename N::T>& lp,
                                                    const NestColArgs<typename N::T>& a, NestChunk& ck) {
     NestColGeo g;
@@ -699,8 +689,8 @@ __device__ __forceinline__ NestColGeo nest_col_geo(const LineParams<typename N::
     g.ci = g.rank * a.slots + g.slot;
     g.live = g.slot < a.slots && g.ci < a.cut.nc;
     if (!g.live) g.ci = 0;
-    ck.cnt = !g.live ? 0 : (!RAG || g.ci < a.cut.rem) ? K : K - S;
-    g.start = RAG ? g.ci * (K - S) + S * min(g.ci, a.cut.rem) : g.ci * K;
+    ck.cnt = !g.live ? 0 : (!RAG || g.ci < a.cut.rem) ? K : K - 1;
+    g.start = RAG ? g.ci * (K - 1) + min(g.ci, a.cut.rem) : g.ci * K;
     const int col = ((blockIdx.x << a.lcp) + g.cpi) * N::W;
     g.on = g.live && col < a.ncols;
     g.both = col + 1 < a.ncols;
@@ -711,7 +701,7 @@ __device__ __forceinline__ NestColGeo nest_col_geo(const LineParams<typename N::
     return g;
 }
 
-template <class N, int K, int S, bool RAG, class SH>
+template <class N, int K, bool RAG, class SH>
 __device__ __forceinline__ NestColScan<typename N::V, typename N::T> nest_col_scan_setup(
     const LineParams<typename N::T>& lp, const NestColArgs<typename N::T>& a, const NestColGeo& g, const NestChunk& ck,
     typename N::V* ex, typename N::T* dec, SH& sh) {
@@ -720,7 +710,7 @@ __device__ __forceinline__ NestColScan<typename N::V, typename N::T> nest_col_sc
     // first node of block r of the cluster
     auto first = [&](int r) {
         const int ch = min(r * a.slots, a.cut.nc);
-        return RAG ? ch * (K - S) + S * min(ch, a.cut.rem) : ch * K;
+        return RAG ? ch * (K - 1) + min(ch, a.cut.rem) : ch * K;
     };
     dec[0] = dev_exp(-lp.nu * T(max(g.start - m, 0)));
     dec[g.nt] = dev_exp(-lp.nu * T(max(lp.n - g.start - ck.cnt - m, 0)));
@@ -814,13 +804,13 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     using V = typename N::V;
     using T = typename N::T;
     constexpr bool RAG = FORM == 2;
-    constexpr int K = kNestColK, H = M / 2, S = 1, NF = MODE == NEST_COPY ? 1 : 2;
+    constexpr int K = kNestColK, H = M / 2, NF = MODE == NEST_COPY ? 1 : 2;
     // per thread in shared memory: arrays 0 = field 0 (w, then s), 1 = field 1 (G, then b), 2 = w, then
     // the ends of field 1's window
     extern __shared__ __align__(16) unsigned char nest_sm[];
     __shared__ NestColShared<N, NF> sh;
     NestChunk ck;
-    const NestColGeo g = nest_col_geo<N, K, S, RAG>(lp, a, ck);
+    const NestColGeo g = nest_col_geo<N, K, RAG>(lp, a, ck);
     const int nt = g.nt;
     const V* all = reinterpret_cast<const V*>(nest_sm);
     constexpr int NA = MODE == NEST_COPY ? 1 : 3, PITCH = nest_col_pitch<K, M, NA>();
@@ -881,7 +871,7 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     }
     V* ex = reinterpret_cast<V*>(nest_sm) + PITCH * nt;
     T* dec = reinterpret_cast<T*>(ex + ((2 * NF) << a.lcp) * (a.slots + 4)) + threadIdx.x;
-    const NestColScan<V, T> c = nest_col_scan_setup<N, K, S, RAG>(lp, a, g, ck, ex, dec, sh);
+    const NestColScan<V, T> c = nest_col_scan_setup<N, K, RAG>(lp, a, g, ck, ex, dec, sh);
 
 #pragma unroll 1
     for (int level = MODE == NEST_COPY && a.single ? 1 : 0; level < 2; ++level) {
@@ -895,7 +885,7 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
             const int pr = pin || !g.live ? g.rank : g.rank > 0 ? g.rank - 1 : a.C - 1;
             const int fr = fin || !g.live ? g.rank : g.ci < nc - 1 ? g.rank + 1 : 0;
             const int ps = pin ? g.slot - 1 : g.rank > 0 ? a.slots - 1 : last, fs = fin ? g.slot + 1 : 0;
-            const int pcnt = (!RAG || (g.ci > 0 ? g.ci - 1 : nc - 1) < a.cut.rem) ? K : K - S;
+            const int pcnt = (!RAG || (g.ci > 0 ? g.ci - 1 : nc - 1) < a.cut.rem) ? K : K - 1;
             const V* pe = all + ((ps << a.lcp) + g.cpi) * PITCH + (pcnt - H);
             const V* fe = all + ((fs << a.lcp) + g.cpi) * PITCH;
 #pragma unroll
@@ -907,7 +897,7 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
                     l[h] = pr == g.rank ? *lp_ : nest_from_bits(nest_ld_cluster(lp_, pr), V());
                     r[h] = fr == g.rank ? *rp : nest_from_bits(nest_ld_cluster(rp, fr), V());
                 }
-                if (RAG && ck.cnt == K - S) {
+                if (RAG && ck.cnt == K - 1) {
                     arr(q, K - 1) = r[0];
 #pragma unroll
                     for (int h = 0; h + 1 < H; ++h) r[h] = r[h + 1];
@@ -937,7 +927,7 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
         for (int q = 0; q < NF; ++q) {
             window(q);
             V aL, aR;
-            nest_chunk_agg<N, K, M, S, RAG>(lp, w, a.pw, ck, x, aL, aR);
+            nest_chunk_agg<N, K, M, RAG>(lp, w, a.pw, ck, x, aL, aR);
             if (g.slot < a.slots) {
                 V* e = ex + 2 * ((q << a.lcp) + g.cpi) * (a.slots + 4) + g.slot;
                 e[0] = aL;
@@ -975,7 +965,7 @@ nest_cols_kernel(const __grid_constant__ LineParams<typename N::T> lp,
             }
         };
         auto finish = [&](int q) {
-            nest_chunk_finish<N, K, M, S, RAG>(lp, w, ck, x, nest_col_carry<N, NF>(lp, c, sh, q, 0),
+            nest_chunk_finish<N, K, M, RAG>(lp, w, ck, x, nest_col_carry<N, NF>(lp, c, sh, q, 0),
                                                nest_col_carry<N, NF>(lp, c, sh, q, 1),
                                                [&](int dir) { return nest_col_end<N, NF>(lp, c, sh, q, dir); }, out);
         };
@@ -1049,12 +1039,12 @@ nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     using V = typename N::V;
     using T = typename N::T;
     constexpr bool RAG = FORM == 2;
-    constexpr int K = kNestColK, H = M / 2, S = 1, NF = 3, PITCH = nest_col3_pitch<K, M>();
+    constexpr int K = kNestColK, H = M / 2, NF = 3, PITCH = nest_col3_pitch<K, M>();
     // per thread: three arrays of the chunk's nodes, then the ends of the windows of fields 1 and 2
     extern __shared__ __align__(16) unsigned char nest_sm[];
     __shared__ NestColShared<N, NF> sh;
     NestChunk ck;
-    const NestColGeo g = nest_col_geo<N, K, S, RAG>(lp, a, ck);
+    const NestColGeo g = nest_col_geo<N, K, RAG>(lp, a, ck);
     const V* all = reinterpret_cast<const V*>(nest_sm);
     V* own = reinterpret_cast<V*>(nest_sm) + threadIdx.x * PITCH;
     auto arr = [&](int f, int k) -> V& { return own[f * K + k]; };
@@ -1099,7 +1089,7 @@ nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
     }
     V* ex = reinterpret_cast<V*>(nest_sm) + PITCH * g.nt;
     T* dec = reinterpret_cast<T*>(ex + ((2 * NF) << a.lcp) * (a.slots + 4)) + threadIdx.x;
-    const NestColScan<V, T> c = nest_col_scan_setup<N, K, S, RAG>(lp, a, g, ck, ex, dec, sh);
+    const NestColScan<V, T> c = nest_col_scan_setup<N, K, RAG>(lp, a, g, ck, ex, dec, sh);
 
 #pragma unroll 1
     for (int level = 0; level < 2; ++level) {
@@ -1112,7 +1102,7 @@ nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
             const int pr = pin || !g.live ? g.rank : g.rank > 0 ? g.rank - 1 : a.C - 1;
             const int fr = fin || !g.live ? g.rank : g.ci < nc - 1 ? g.rank + 1 : 0;
             const int ps = pin ? g.slot - 1 : g.rank > 0 ? a.slots - 1 : last, fs = fin ? g.slot + 1 : 0;
-            const int pcnt = (!RAG || (g.ci > 0 ? g.ci - 1 : nc - 1) < a.cut.rem) ? K : K - S;
+            const int pcnt = (!RAG || (g.ci > 0 ? g.ci - 1 : nc - 1) < a.cut.rem) ? K : K - 1;
             const V* pe = all + ((ps << a.lcp) + g.cpi) * PITCH + (pcnt - H);
             const V* fe = all + ((fs << a.lcp) + g.cpi) * PITCH;
 #pragma unroll
@@ -1124,7 +1114,7 @@ nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
                     l[h] = pr == g.rank ? *lq : nest_from_bits(nest_ld_cluster(lq, pr), V());
                     r[h] = fr == g.rank ? *rq : nest_from_bits(nest_ld_cluster(rq, fr), V());
                 }
-                if (RAG && ck.cnt == K - S) {
+                if (RAG && ck.cnt == K - 1) {
                     arr(q, K - 1) = r[0];
 #pragma unroll
                     for (int h = 0; h + 1 < H; ++h) r[h] = r[h + 1];
@@ -1136,7 +1126,7 @@ nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
         for (int q = 0; q < NF; ++q) {
             window(q);
             V aL, aR;
-            nest_chunk_agg<N, K, M, S, RAG>(lp, w, a.pw, ck, x, aL, aR);
+            nest_chunk_agg<N, K, M, RAG>(lp, w, a.pw, ck, x, aL, aR);
             if (g.slot < a.slots) {
                 V* e = ex + 2 * ((q << a.lcp) + g.cpi) * (a.slots + 4) + g.slot;
                 e[0] = aL;
@@ -1156,7 +1146,7 @@ nest_cols3_kernel(const __grid_constant__ LineParams<typename N::T> lp,
         V out[K];
         auto finish = [&](int q) {
             window(q);
-            nest_chunk_finish<N, K, M, S, RAG>(lp, w, ck, x, nest_col_carry<N, NF>(lp, c, sh, q, 0),
+            nest_chunk_finish<N, K, M, RAG>(lp, w, ck, x, nest_col_carry<N, NF>(lp, c, sh, q, 0),
                                                nest_col_carry<N, NF>(lp, c, sh, q, 1),
                                                [&](int dir) { return nest_col_end<N, NF>(lp, c, sh, q, dir); }, out);
         };

@@ -1,5 +1,5 @@
 // Launch layer of the nested passes (nest.cuh, nest_rows.cuh), one quadrature order per translation
-// unit (nest_m2.cu, nest_m4.cu, nest_m6.cu).
+// unit and precision (nest_f32_m2.cu to nest_f64_m6.cu).
 #pragma once
 
 #include <cmath>

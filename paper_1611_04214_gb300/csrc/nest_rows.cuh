@@ -149,7 +149,7 @@ __device__ __forceinline__ void nest_row_scan(const LineParams<typename N::T>& l
 }
 
 // Edge values of the neighbouring chunks of the line (wrapped; a low half continues in the high half).
-template <class N, int K, int M, int S, bool RAG, bool WARP, int KM>
+template <class N, int K, int M, bool RAG, bool WARP, int KM>
 __device__ __forceinline__ void nest_row_halo(const NestRowScan<typename N::T>& c, int nc, int cnt,
                                               typename N::V* edge, int TL, typename N::V (&x)[KM]) {
     using V = typename N::V;
@@ -159,7 +159,7 @@ __device__ __forceinline__ void nest_row_halo(const NestRowScan<typename N::T>& 
 #pragma unroll
     for (int h = 0; h < H; ++h) {
         V e = x[H + K - H + h];
-        if (RAG && cnt != K) e = x[H + K - S - H + h];
+        if (RAG && cnt != K) e = x[H + K - 1 - H + h];
         if constexpr (WARP) {
             const int base = c.lane - tl;
             const int pl = base + (tl > 0 ? tl - 1 : nc - 1), fl = base + (tl < nc - 1 ? tl + 1 : 0);
@@ -186,7 +186,7 @@ __device__ __forceinline__ void nest_row_halo(const NestRowScan<typename N::T>& 
             if (tl == nc - 1) r[h] = N::swap(r[h]);
         }
     }
-    nest_set_halo<N, K, M, S, RAG>(cnt, l, r, x);
+    nest_set_halo<N, K, M, RAG>(cnt, l, r, x);
 }
 
 // Nodes p.. of one half line (float4 chunks), or of a scalar line.
@@ -259,7 +259,6 @@ template <class N, int K, bool RAG, bool WARP>
 __device__ __forceinline__ NestRowThread<N> nest_row_thread(const LineParams<typename N::T>& lp,
                                                             const NestRowLayout<typename N::T>& a) {
     using T = typename N::T;
-    constexpr int S = 1;
     NestRowThread<N> g;
     NestRowScan<T>& c = g.c;
     c.lane = threadIdx.x & 31;
@@ -276,8 +275,8 @@ __device__ __forceinline__ NestRowThread<N> nest_row_thread(const LineParams<typ
     const bool live = c.tl < a.cut.nc;
     g.on = live && g.line < a.nlines;
     const int ci = live ? c.tl : 0;
-    g.ck.cnt = !live ? 0 : (!RAG || ci < a.cut.rem) ? K : K - S;
-    g.start = RAG ? ci * (K - S) + S * min(ci, a.cut.rem) : ci * K;
+    g.ck.cnt = !live ? 0 : (!RAG || ci < a.cut.rem) ? K : K - 1;
+    g.start = RAG ? ci * (K - 1) + min(ci, a.cut.rem) : ci * K;
     const bool periodic = lp.bc == BC_PERIODIC;
     g.ck.mA = live && !periodic && ci == 0 ? 1 : 0;
     g.ck.mB = live && !periodic && ci == a.cut.nc - 1 ? N::W : 0;
@@ -347,10 +346,10 @@ __device__ __forceinline__ void nest_row_inverse(const LineParams<typename N::T>
                                                  typename N::V (&out)[K]) {
     using V = typename N::V;
     V aL, aR, cL, cR, XL, XR;
-    nest_row_halo<N, K, M, 1, RAG, WARP>(g.c, a.cut.nc, g.ck.cnt, edge, a.TL, x);
-    nest_chunk_agg<N, K, M, 1, RAG>(lp, w, a.pw, g.ck, x, aL, aR);
+    nest_row_halo<N, K, M, RAG, WARP>(g.c, a.cut.nc, g.ck.cnt, edge, a.TL, x);
+    nest_chunk_agg<N, K, M, RAG>(lp, w, a.pw, g.ck, x, aL, aR);
     nest_row_scan<N, WARP>(lp, g.c, sh, aL, aR, cL, cR, XL, XR);
-    nest_chunk_finish<N, K, M, 1, RAG>(lp, w, g.ck, x, cL, cR, [&](int dir) { return dir ? XR : XL; }, out);
+    nest_chunk_finish<N, K, M, RAG>(lp, w, g.ck, x, cL, cR, [&](int dir) { return dir ? XR : XL; }, out);
 }
 
 // value(k), the thread's k-th node, to a field.
