@@ -189,18 +189,20 @@ struct RedAcc {
     T vmax;   // max |w_new| (stored variable)
 };
 
-// The larger of two absolute values; a NaN on either side stays (fmax would drop it, and an iterate that has
-// overflowed into NaN throughout would leave a residual of zero).  FP64 by bit patterns: non-negative doubles order
-// like them, NaN above infinity, and the integer units are idle beside this part's FP64 units.  (fabs may leave the
-// sign of a NaN set: it is masked here.)
+// The larger of a maximum so far and one more absolute value; a NaN stays (fmax would drop it, and an iterate that has
+// overflowed into NaN throughout would leave a residual of zero).  FP64 by unsigned bit patterns: non-negative
+// doubles order like them, a NaN of either sign above infinity (fabs may leave its sign set), and the integer units
+// are idle beside this part's FP64 units.
 __device__ __forceinline__ float abs_max(float a, float b) {
     float r;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
 }
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+    return static_cast<unsigned long long>(__double_as_longlong(x));
+}
 __device__ __forceinline__ double abs_max(double a, double b) {
-    constexpr long long kAbs = 0x7fffffffffffffffLL;
-    return __longlong_as_double(max(__double_as_longlong(a) & kAbs, __double_as_longlong(b) & kAbs));
+    return __longlong_as_double(static_cast<long long>(max(abs_bits(a), abs_bits(b))));
 }
 
 template <typename T>
@@ -517,16 +519,16 @@ struct Op1aV : OpBase<T> {
     }
 };
 
-// Block-wide max of the two residual values, then one atomic max per block on the
-// bit patterns (non-negative doubles order like their unsigned bits).
+// Block-wide max of the two residual values and one atomic max per block, on the bit patterns
+// (non-negative doubles order like their unsigned bits, a NaN above infinity).
 template <typename T>
 __device__ __forceinline__ void block_reduce_store(RedAcc<T> r, unsigned long long* slots) {
-    __shared__ double s_d[32], s_v[32];
-    double a = static_cast<double>(r.dmax), b = static_cast<double>(r.vmax);
+    __shared__ unsigned long long s_d[32], s_v[32];
+    unsigned long long a = abs_bits(static_cast<double>(r.dmax)), b = abs_bits(static_cast<double>(r.vmax));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        a = abs_max(a, __shfl_xor_sync(kFull, a, o));
-        b = abs_max(b, __shfl_xor_sync(kFull, b, o));
+        a = max(a, __shfl_xor_sync(kFull, a, o));
+        b = max(b, __shfl_xor_sync(kFull, b, o));
     }
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int nthreads = blockDim.x * blockDim.y;
@@ -538,16 +540,16 @@ __device__ __forceinline__ void block_reduce_store(RedAcc<T> r, unsigned long lo
     __syncthreads();
     if (warp == 0) {
         const int nw = (nthreads + 31) >> 5;
-        a = lane < nw ? s_d[lane] : 0.0;
-        b = lane < nw ? s_v[lane] : 0.0;
+        a = lane < nw ? s_d[lane] : 0ull;
+        b = lane < nw ? s_v[lane] : 0ull;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            a = abs_max(a, __shfl_xor_sync(kFull, a, o));
-            b = abs_max(b, __shfl_xor_sync(kFull, b, o));
+            a = max(a, __shfl_xor_sync(kFull, a, o));
+            b = max(b, __shfl_xor_sync(kFull, b, o));
         }
         if (lane == 0) {
-            atomicMax(&slots[0], static_cast<unsigned long long>(__double_as_longlong(a)));
-            atomicMax(&slots[1], static_cast<unsigned long long>(__double_as_longlong(b)));
+            atomicMax(&slots[0], a);
+            atomicMax(&slots[1], b);
         }
     }
 }
