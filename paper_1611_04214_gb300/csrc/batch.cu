@@ -131,7 +131,7 @@ rows_batch_kernel(const RowItem* __restrict__ items, int nitems, const Inst* __r
         op.ls = in.nx;
         op.ps = 1;
         rows_body<float, M, kRowK, Op>(slp, op, in.ny, it.tl_log2, it.lpb, it.pitch, it.line0,
-                                       reinterpret_cast<float*>(sm_rows_batch), red + 2 * it.inst);
+                                       reinterpret_cast<float*>(sm_rows_batch), red + kRedSlots * it.inst);
     };
     if constexpr (!kLoop) {
         body(blockIdx.x);
@@ -214,7 +214,7 @@ cols_final_batch_kernel(const ColItem* __restrict__ items, int nitems, const Ins
         op.ls = 1;
         op.ps = in.nx;
         cols_final_body<float, M, kColKY, kColWY, Op>(slp, op, in.nx, carL + in.soff, carR + in.soff, in.tiles,
-                                                      it.strip, it.tile, red + 2 * it.inst);
+                                                      it.strip, it.tile, red + kRedSlots * it.inst);
     };
     if constexpr (!kLoop) {
         body(blockIdx.x);
@@ -237,8 +237,7 @@ __global__ void loop_init_batch_kernel(LoopState* ls, unsigned long long* red, i
         s.res = s.best;
         s.tol_used = 0.0;
         ls[i] = s;
-        red[2 * i] = 0ull;
-        red[2 * i + 1] = 0ull;
+        for (int k = 0; k < kRedSlots; ++k) red[kRedSlots * i + k] = 0ull;
         done[i] = 0;
     }
 }
@@ -290,8 +289,9 @@ __global__ void loop_check_batch_kernel(cudaGraphConditionalHandle h, LoopState*
     int active = 0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         if (!done[i]) {
-            const double res = __longlong_as_double(static_cast<long long>(red[2 * i]));
-            const double wmax = __longlong_as_double(static_cast<long long>(red[2 * i + 1]));
+            const double res = __longlong_as_double(static_cast<long long>(red[kRedSlots * i]));
+            const double wmax = __longlong_as_double(static_cast<long long>(red[kRedSlots * i + 1]));
+            const bool bad = red[kRedSlots * i + 2] != 0;
             LoopState s = ls[i];
             s.k += 1;
             const double ulp = wmax * 5.9604644775390625e-08;   // 2^-24 max|w|
@@ -308,16 +308,15 @@ __global__ void loop_check_batch_kernel(cudaGraphConditionalHandle h, LoopState*
                 conv = true;
                 tol_used = res;
             }
-            s.res = res;
-            s.tol_used = tol_used;
-            s.converged = conv ? 1 : 0;
             stop = stop || conv || s.k >= max_iter;
+            s.res = bad ? nan("") : res;
+            s.tol_used = tol_used;
+            s.converged = conv && !bad ? 1 : 0;
             s.done = stop ? 1 : 0;
             ls[i] = s;
             done[i] = s.done;
         }
-        red[2 * i] = 0ull;
-        red[2 * i + 1] = 0ull;
+        for (int k = 0; k < kRedSlots; ++k) red[kRedSlots * i + k] = 0ull;
         active |= done[i] ? 0 : 1;
     }
     active = __syncthreads_or(active);
@@ -358,7 +357,7 @@ struct molt_batch {
     int* done = nullptr;                // [count]
     int* active = nullptr;              // [1] (host-driven loop)
     LoopState* ls = nullptr;            // [count]
-    unsigned long long* red = nullptr;  // [count][2]
+    unsigned long long* red = nullptr;  // [count][kRedSlots]
     RowItem* rows = nullptr;
     ColItem* cols = nullptr;
     CarryItem* carry[2] = {nullptr, nullptr};
@@ -843,7 +842,7 @@ molt_status molt_batch_create(molt_batch** out, int count, const molt_instance* 
     const size_t nt = static_cast<size_t>(b->total), ns = static_cast<size_t>(b->scratch);
     bool ok = balloc(b, &b->inst, count) && balloc(b, &b->lps, 4 * static_cast<size_t>(count)) &&
               balloc(b, &b->stages, count) && balloc(b, &b->done, count) && balloc(b, &b->active, 1) &&
-              balloc(b, &b->ls, count) && balloc(b, &b->red, 2 * static_cast<size_t>(count)) &&
+              balloc(b, &b->ls, count) && balloc(b, &b->red, molt::kRedSlots * static_cast<size_t>(count)) &&
               balloc(b, &b->rows, rows.size()) && balloc(b, &b->cols, cols.size()) &&
               balloc(b, &b->carry[0], carry[0].size()) && balloc(b, &b->carry[1], carry[1].size()) &&
               balloc(b, &b->w, nt) && balloc(b, &b->r, nt) && balloc(b, &b->Y, nt) && balloc(b, &b->wprev, nt) &&

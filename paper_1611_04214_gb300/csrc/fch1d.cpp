@@ -74,7 +74,7 @@ struct Fch1d final : molt_fch1d {
         for (T** q : {&v, &vn, &vnew, &h2vn, &lap, &f, &pp, &hv, &dv, &hdv, &df, &hdf, &dp, &hdp, &z, &zero})
             if (!alloc(q)) return false;
         void* m = nullptr;
-        if (cudaMalloc(&m, 2 * sizeof(unsigned long long)) != cudaSuccess) return false;
+        if (cudaMalloc(&m, molt::kRedSlots * sizeof(unsigned long long)) != cudaSuccess) return false;
         allocs.push_back(m);
         red = static_cast<unsigned long long*>(m);
         return cudaMemset(zero, 0, n * sizeof(T)) == cudaSuccess &&
@@ -93,14 +93,16 @@ struct Fch1d final : molt_fch1d {
         return molt::lincomb<T>(out, static_cast<long long>(n), x0, c0, x1, c1, x2, c2, x3, c3, c4, st, &launches);
     }
 
-    double read_max(const T* a, const T* b, cudaStream_t st, cudaError_t* e) {
+    // max |a - b| over the values that are numbers; *bad: whether any was a NaN.
+    double read_max(const T* a, const T* b, cudaStream_t st, cudaError_t* e, bool* bad) {
         double r = 0.0;
         if ((*e = molt::max_abs_diff<T>(a, b, static_cast<long long>(n), red, st)) != cudaSuccess ||
-            (*e = cudaMemcpyAsync(red_host, red, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
+            (*e = cudaMemcpyAsync(red_host, red, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
                 cudaSuccess ||
             (*e = cudaStreamSynchronize(st)) != cudaSuccess)
             return 0.0;
         std::memcpy(&r, red_host, sizeof(double));
+        *bad = red_host[1] != 0;
         launches += 1;
         return r;
     }
@@ -146,7 +148,7 @@ struct Fch1d final : molt_fch1d {
                 return fail_f(MOLT_ERR_CUDA, std::string("sixth-order step load: ") + cudaGetErrorString(e));
         double res = INFINITY, best = INFINITY, tol_used = p.tol;
         int k = 0, stall = 0;
-        bool converged = false;
+        bool converged = false, bad = false, bad_max = false;   // bad: the last iteration left a NaN (kRedSlots)
         const bool fp32 = sizeof(T) == 4;
         if (fused()) {
             // one kernel per iteration (nest_fch_kernel), the loop on the device: 16384 lines of 1024 nodes, FP32, M = 6:
@@ -181,7 +183,7 @@ struct Fch1d final : molt_fch1d {
                 (e = H(lp, z, vnew, st)) != cudaSuccess ||
                 (e = lin(lap, vnew, 1.0 / a, z, -1.0 / a, nullptr, 0, nullptr, 0, 0.0, st)) != cudaSuccess)
                 return fail_f(MOLT_ERR_CUDA, std::string("sixth-order iteration: ") + cudaGetErrorString(e));
-            res = read_max(vnew, v, st, &e);
+            res = read_max(vnew, v, st, &e, &bad);
             if (e != cudaSuccess) return fail_f(MOLT_ERR_CUDA, std::string("residual: ") + cudaGetErrorString(e));
             std::swap(v, vnew);
             if (!std::isfinite(res)) break;
@@ -189,7 +191,7 @@ struct Fch1d final : molt_fch1d {
             tol_used = p.tol;
             if (fp32) {
                 // 2 ulp of max|v| (against the zero field): the FP32 rounding floor of the iterate
-                const double vmax = read_max(v, zero, st, &e);
+                const double vmax = read_max(v, zero, st, &e, &bad_max);
                 if (e != cudaSuccess) return fail_f(MOLT_ERR_CUDA, std::string("residual: ") + cudaGetErrorString(e));
                 ulp = std::ldexp(1.0, -24) * vmax;
                 tol_used = std::max(p.tol, 2.0 * ulp);
@@ -207,7 +209,7 @@ struct Fch1d final : molt_fch1d {
                 break;
             }
         }
-        return finish(u, converged, k, res, tol_used, st, info);
+        return finish(u, converged, k, bad ? NAN : res, tol_used, st, info);
     }
 
     // The iterate back to u, the step's outcome.
@@ -217,6 +219,7 @@ struct Fch1d final : molt_fch1d {
         if ((e = lin(u, v, 1.0, nullptr, 0, nullptr, 0, nullptr, 0, -1.0, st)) != cudaSuccess)
             return fail_f(MOLT_ERR_CUDA, std::string("sixth-order store: ") + cudaGetErrorString(e));
         const int it = converged ? k : std::min(k, p.max_iter);
+        if (!std::isfinite(res)) converged = false;
         if (info) {
             info->status = converged ? MOLT_OK : MOLT_ERR_NOT_CONVERGED;
             info->stages = 1;

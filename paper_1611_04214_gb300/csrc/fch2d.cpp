@@ -103,7 +103,7 @@ struct Fch2d final : molt_fch2d {
         cs.capacity_lines = nx;
         cs.capacity_fields = 2;
         if (!alloc(&cs.aggL, sc) || !alloc(&cs.aggR, sc) || !alloc(&cs.carL, sc) || !alloc(&cs.carR, sc) ||
-            !alloc(&red, 4) || !alloc(&status, 1))
+            !alloc(&red, 2 * molt::kRedSlots) || !alloc(&status, 1))
             return false;
         cs.status = status;
         if (cudaMemset(zero, 0, n * sizeof(T)) != cudaSuccess || cudaMemset(status, 0, sizeof(unsigned)) != cudaSuccess ||
@@ -147,16 +147,18 @@ struct Fch2d final : molt_fch2d {
         return lin(xw, vout, 1.0, hx, -1.0, hy, -1.0, w, 1.0, st);
     }
 
-    // max |a - b| (FP64 bits through the reduction word) and the column kernels' wait status
-    double read_max(const T* a, const T* b, cudaStream_t st, cudaError_t* e) {
+    // max |a - b| over the values that are numbers (FP64 bits through the reduction words; *bad: whether any was a NaN)
+    // and the column kernels' wait status
+    double read_max(const T* a, const T* b, cudaStream_t st, cudaError_t* e, bool* bad) {
         double r = 0.0;
         if ((*e = molt::max_abs_diff<T>(a, b, static_cast<long long>(n), red, st)) != cudaSuccess ||
-            (*e = cudaMemcpyAsync(red_host, red, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
+            (*e = cudaMemcpyAsync(red_host, red, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
                 cudaSuccess ||
             (*e = cudaMemcpyAsync(status_host, status, sizeof(unsigned), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
             (*e = cudaStreamSynchronize(st)) != cudaSuccess)
             return 0.0;
         std::memcpy(&r, red_host, sizeof(double));
+        *bad = red_host[1] != 0;
         launches += 1;
         return r;
     }
@@ -196,7 +198,7 @@ struct Fch2d final : molt_fch2d {
         molt::NestCols<T> y = cols(s1, aa);
         y.in1 = s2, y.in2 = s3, y.U = ee, y.Y = dd, y.o1 = cc, y.o2 = tt;
         molt::NestRows<T> x;
-        x.A = aa, x.B = cc, x.E = tt, x.w = W, x.nlines = ny, x.red = red + 2;   // (the residual is that of v)
+        x.A = aa, x.B = cc, x.E = tt, x.w = W, x.nlines = ny, x.red = red + molt::kRedSlots;   // (the residual is that of v)
         cudaError_t e;
         if ((e = molt::nest_cols<T>(lp.y, molt::NEST_FCH2, y, st, nullptr)) != cudaSuccess ||
             (e = molt::nest_rows<T>(lp.x, molt::NEST_ROW_PASS, x, st, nullptr)) != cudaSuccess)
@@ -235,7 +237,7 @@ molt_status Fch2d<T>::step(void* uv, double dt, cudaStream_t st, molt_step_info*
         return fail2(MOLT_ERR_CUDA, std::string("sixth-order 2D step load: ") + cudaGetErrorString(e));
     double res = INFINITY, best = INFINITY, tol_used = p.tol;
     int k = 0, stall = 0;
-    bool converged = false;
+    bool converged = false, bad = false, bad_max = false;   // bad: the last iteration left a NaN (kRedSlots)
     const bool fp32 = sizeof(T) == 4;
     for (k = 1; k <= p.max_iter; ++k) {
         if ((e = molt::fch_pointwise<T>(static_cast<long long>(n), v, lap, eps * eps, eta * eps * eps, f, pp, st,
@@ -261,7 +263,7 @@ molt_status Fch2d<T>::step(void* uv, double dt, cudaStream_t st, molt_step_info*
             (e = lin(Wn, tt, 1.0, m2vn, 1.0, nullptr, 0.0, nullptr, 0.0, st)) != cudaSuccess ||
             (e = from_w(lp, Wn, vnew, a, st)) != cudaSuccess)
             return fail2(MOLT_ERR_CUDA, std::string("sixth-order 2D iteration: ") + cudaGetErrorString(e));
-        res = read_max(vnew, v, st, &e);
+        res = read_max(vnew, v, st, &e, &bad);
         if (e != cudaSuccess) return fail2(MOLT_ERR_CUDA, std::string("residual: ") + cudaGetErrorString(e));
         if (*status_host)
             return fail2(MOLT_ERR_CUDA, "a column kernel's bounded wait for a tile copy ran out; the field is incomplete");
@@ -272,7 +274,7 @@ molt_status Fch2d<T>::step(void* uv, double dt, cudaStream_t st, molt_step_info*
         tol_used = p.tol;
         if (fp32) {
             // 2 ulp of max|v| (against the zero field): the FP32 rounding floor of the iterate
-            const double vmax = read_max(v, zero, st, &e);
+            const double vmax = read_max(v, zero, st, &e, &bad_max);
             if (e != cudaSuccess) return fail2(MOLT_ERR_CUDA, std::string("residual: ") + cudaGetErrorString(e));
             ulp = std::ldexp(1.0, -24) * vmax;
             tol_used = std::max(p.tol, 2.0 * ulp);
@@ -290,7 +292,7 @@ molt_status Fch2d<T>::step(void* uv, double dt, cudaStream_t st, molt_step_info*
             break;
         }
     }
-    return finish(u, converged, k, res, tol_used, st, info);
+    return finish(u, converged, k, bad ? NAN : res, tol_used, st, info);
 }
 
 template <typename T>
@@ -328,6 +330,7 @@ molt_status Fch2d<T>::finish(T* u, bool converged, int k, double res, double tol
                               &launches)) != cudaSuccess)
         return fail2(MOLT_ERR_CUDA, std::string("sixth-order 2D store: ") + cudaGetErrorString(e));
     const int it = converged ? k : std::min(k, p.max_iter);
+    if (!std::isfinite(res)) converged = false;
     if (info) {
         info->status = converged ? MOLT_OK : MOLT_ERR_NOT_CONVERGED;
         info->stages = 1;

@@ -29,14 +29,17 @@ __global__ void loop_init_kernel(LoopState* ls, unsigned long long* red) {
     ls->tol_used = 0.0;
     red[0] = 0ull;
     red[1] = 0ull;
+    red[2] = 0ull;
 }
 
 __global__ void loop_check_kernel(cudaGraphConditionalHandle h, LoopState* ls, unsigned long long* red,
                                   double tol, int max_iter, int fp32) {
     const double res = __longlong_as_double(static_cast<long long>(red[0]));
     const double wmax = __longlong_as_double(static_cast<long long>(red[1]));
+    const bool bad = red[2] != 0;
     red[0] = 0ull;
     red[1] = 0ull;
+    red[2] = 0ull;
     const int k = ls->k + 1;
     ls->k = k;
     const double ulp = wmax * 5.9604644775390625e-08;       // 2^-24 max|w|
@@ -53,10 +56,10 @@ __global__ void loop_check_kernel(cudaGraphConditionalHandle h, LoopState* ls, u
         conv = true;
         tol_used = res;
     }
-    ls->res = res;
-    ls->tol_used = tol_used;
-    ls->converged = conv ? 1 : 0;
     stop = stop || conv || k >= max_iter;
+    ls->res = bad ? nan("") : res;
+    ls->tol_used = tol_used;
+    ls->converged = conv && !bad ? 1 : 0;
     ls->done = stop ? 1 : 0;
     cudaGraphSetConditional(h, stop ? 0u : 1u);
 }

@@ -922,17 +922,22 @@ namespace detail {
 // (for the nearby iterates a residual compares, the difference is exact), and the loop stays a
 // memory stream instead of an FP64 one.  The thread's max is widened to FP64 for the combine; the
 // non-negative FP64 bit patterns order like the values, so blocks combine by an integer atomicMax
-// on *out (zeroed by the caller).
+// on *out (zeroed by the caller).  A NaN is left out of the maximum and sets out[1].
 template <typename T>
 __global__ void max_abs_diff_kernel(const T* __restrict__ a, const T* __restrict__ b, long long n,
                                     unsigned long long* out) {
     T mt = T(0);
+    bool bad = false;
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-         i += static_cast<long long>(gridDim.x) * blockDim.x)
-        mt = abs_max(mt, fabs(a[i] - b[i]));
+         i += static_cast<long long>(gridDim.x) * blockDim.x) {
+        const T x = fabs(a[i] - b[i]);
+        mt = fmax(mt, x);
+        bad |= x != x;
+    }
+    if (__any_sync(kFull, bad) && (threadIdx.x & 31) == 0) atomicMax(out + 1, 1ull);
     double m = static_cast<double>(mt);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = abs_max(m, __shfl_xor_sync(kFull, m, o));
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(kFull, m, o));
     __shared__ double s[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) s[warp] = m;
@@ -940,7 +945,7 @@ __global__ void max_abs_diff_kernel(const T* __restrict__ a, const T* __restrict
     if (warp == 0) {
         m = lane < static_cast<int>(blockDim.x >> 5) ? s[lane] : 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = abs_max(m, __shfl_xor_sync(kFull, m, o));
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(kFull, m, o));
         if (lane == 0) atomicMax(out, static_cast<unsigned long long>(__double_as_longlong(m)));
     }
 }
@@ -949,7 +954,7 @@ __global__ void max_abs_diff_kernel(const T* __restrict__ a, const T* __restrict
 
 template <typename T>
 cudaError_t max_abs_diff(const T* a, const T* b, long long n, unsigned long long* out, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), st);
+    cudaError_t e = cudaMemsetAsync(out, 0, 2 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     detail::max_abs_diff_kernel<T><<<detail::kRedBlocks, 256, 0, st>>>(a, b, n, out);
     return cudaGetLastError();

@@ -21,11 +21,11 @@ class LoopGraphs {
         if (red_host_) cudaFreeHost(red_host_);
     }
 
-    // The state words; red: the two residual slots that the iteration's last kernel accumulates into.
+    // The state words; red: the residual words (kRedSlots) that the iteration's last kernel accumulates into.
     bool init() {
         return cudaMalloc(&ls_, sizeof(LoopState)) == cudaSuccess &&
                cudaMallocHost(&host_, sizeof(LoopState)) == cudaSuccess &&
-               cudaMallocHost(&red_host_, 2 * sizeof(unsigned long long)) == cudaSuccess;
+               cudaMallocHost(&red_host_, kRedSlots * sizeof(unsigned long long)) == cudaSuccess;
     }
 
     // Runs the loop of the stage with coefficient `key` on st and waits for it; body(stream) launches one
@@ -84,17 +84,19 @@ class LoopGraphs {
                           LoopState* out) {
         LoopState ls{};
         ls.best = INFINITY;
+        bool out_nan = false;
         while (!ls.done) {
             cudaError_t e;
-            if ((e = cudaMemsetAsync(red, 0, 2 * sizeof(unsigned long long), st)) != cudaSuccess || (e = body(st)) != cudaSuccess ||
-                (e = cudaMemcpyAsync(red_host_, red, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
+            if ((e = cudaMemsetAsync(red, 0, kRedSlots * sizeof(unsigned long long), st)) != cudaSuccess ||
+                (e = body(st)) != cudaSuccess ||
+                (e = cudaMemcpyAsync(red_host_, red, kRedSlots * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
                     cudaSuccess ||
                 (e = cudaStreamSynchronize(st)) != cudaSuccess)
                 return e;
             double wmax;
             std::memcpy(&ls.res, &red_host_[0], sizeof(double));
             std::memcpy(&wmax, &red_host_[1], sizeof(double));
-            // as loop_check: tolerance, FP32 floor of 2 ulp of max|w|, stall at the FP32 noise floor, cap
+            // as loop_check: tolerance, FP32 floor of 2 ulp of max|w|, stall at the FP32 noise floor, cap, NaN
             const double ulp = wmax * 5.9604644775390625e-08;
             ls.tol_used = fp32 ? std::fmax(tol, 2.0 * ulp) : tol;
             ls.k += 1;
@@ -111,8 +113,10 @@ class LoopGraphs {
                 ls.tol_used = ls.res;
             }
             ls.done = stop || ls.converged;
+            out_nan = red_host_[2] != 0;
         }
         *out = ls;
+        if (out_nan) out->converged = 0, out->res = NAN;
         return cudaSuccess;
     }
 

@@ -268,6 +268,11 @@ struct LoopState {
     double tol_used;  // tolerance applied at the last check
 };
 
+// The residual words of an iteration: the bit patterns of max |w_new - w| and max |w_new| over the values that are
+// numbers, and 1 where any was a NaN.  Independent lines go on beside one that has overflowed; an iteration that
+// leaves a NaN never counts as converged.
+constexpr int kRedSlots = 3;
+
 // Reset the loop state and the residual slots (one thread).
 cudaError_t loop_init(LoopState* ls, unsigned long long* red, cudaStream_t st);
 // Read the residual slots, apply the stopping rule of the host loop (tolerance, FP32 floor of

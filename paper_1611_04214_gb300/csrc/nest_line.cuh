@@ -144,7 +144,7 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
     }
     // state of the stopping rule (thread 0)
     double best = __longlong_as_double(0x7ff0000000000000LL), res = best, vmax = 0.0, tol_used = 0.0;
-    int stall = 0, conv = 0, k_it = 0;
+    int stall = 0, conv = 0, k_it = 0, bad = 0;
     for (;;) {
         V gl[K];
 #pragma unroll
@@ -162,23 +162,24 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
         for (int k = 0; k < K; ++k)
             if (k < cnt) {
                 const T nw = y[k] + out[k];
-                dm = abs_max(dm, fabs(nw - w[k]));
+                dm = fmax(dm, fabs(nw - w[k]));
                 vm = abs_max(vm, fabs(nw));
                 w[k] = a.fix && (start + k == 0 || start + k == n - 1) ? a.wall : nw;
             }
+        const bool nan_here = vm != vm;
         dm = nest_warp_max(dm);
-        vm = nest_warp_max(vm);
+        vm = nest_warp_max(nan_here ? T(0) : vm);
         if (g.c.lane == 0) {
             s_max[0][g.c.warp] = dm;
             s_max[1][g.c.warp] = vm;
         }
-        __syncthreads();
+        bad = __syncthreads_or(nan_here);
         if (threadIdx.x == 0) {
-            // as loop_check: tolerance, FP32 floor of 2 ulp of max|w|, stall at the FP32 noise floor, cap
+            // as loop_check: tolerance, FP32 floor of 2 ulp of max|w|, stall at the FP32 noise floor, cap, NaN
             T d = T(0), v = T(0);
             for (int q = 0; q < g.c.nwarps; ++q) {
-                d = abs_max(d, s_max[0][q]);
-                v = abs_max(v, s_max[1][q]);
+                d = fmax(d, s_max[0][q]);
+                v = fmax(v, s_max[1][q]);
             }
             res = static_cast<double>(d);
             vmax = static_cast<double>(v);
@@ -198,6 +199,7 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
                 tol_used = res;
             }
             s_stop = stop || conv || k_it >= a.max_iter;
+            if (bad) conv = 0;
         }
         __syncthreads();
         if (s_stop) break;
@@ -212,12 +214,13 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
         s.done = 1;
         s.converged = conv;
         s.best = best;
-        s.res = res;
+        s.res = bad ? nan("") : res;
         s.tol_used = tol_used;
         *a.ls = s;
         if (a.red) {
             a.red[0] = static_cast<unsigned long long>(__double_as_longlong(res));
             a.red[1] = static_cast<unsigned long long>(__double_as_longlong(vmax));
+            a.red[2] = bad ? 1ull : 0ull;
         }
     }
 }

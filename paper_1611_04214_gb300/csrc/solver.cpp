@@ -284,8 +284,8 @@ struct Solver final : molt_solver {
     T *vw2 = nullptr, *vY2 = nullptr, *vn2 = nullptr, *vp2 = nullptr, *vr2 = nullptr;
     T *vg4 = nullptr, *vg5 = nullptr, *vg6 = nullptr, *vp1 = nullptr;
     molt::ColScratch<T> cs{};
-    unsigned long long* red = nullptr;       // device [2]
-    unsigned long long* red_host = nullptr;  // pinned [2]
+    unsigned long long* red = nullptr;       // device [kRedSlots]
+    unsigned long long* red_host = nullptr;  // pinned [kRedSlots]
     unsigned* wait_status = nullptr;         // device [1]: set by kernels whose bounded waits ran out
     unsigned* wait_status_host = nullptr;    // pinned [1]
     double* dprof = nullptr;                 // device [kProfiles][max(nx, ny)]: Dirichlet offset profiles
@@ -344,7 +344,7 @@ struct Solver final : molt_solver {
         cs.capacity_fields = 2;
         const size_t sc = static_cast<size_t>(2) * tiles * nlines;
         if (!alloc(&cs.aggL, sc) || !alloc(&cs.aggR, sc) || !alloc(&cs.carL, sc) || !alloc(&cs.carR, sc) ||
-            !alloc(&red, 2) || !alloc(&partials, static_cast<size_t>(molt::reduce_blocks())) || !alloc(&result, 1) ||
+            !alloc(&red, molt::kRedSlots) || !alloc(&partials, static_cast<size_t>(molt::reduce_blocks())) || !alloc(&result, 1) ||
             !alloc(&dprof, static_cast<size_t>(kProfiles) * std::max(g.nx, g.ny)))
             return fail(MOLT_ERR_OOM, "device scratch allocation failed");
         if (!alloc(&ls, 1)) return fail(MOLT_ERR_OOM, "device loop state allocation failed");
@@ -352,7 +352,7 @@ struct Solver final : molt_solver {
         if (cudaMemset(wait_status, 0, sizeof(unsigned)) != cudaSuccess)
             return fail(MOLT_ERR_CUDA, "device status initialisation failed");
         cs.status = wait_status;
-        if (cudaMallocHost(&red_host, 2 * sizeof(unsigned long long)) != cudaSuccess ||
+        if (cudaMallocHost(&red_host, molt::kRedSlots * sizeof(unsigned long long)) != cudaSuccess ||
             cudaMallocHost(&result_host, sizeof(double)) != cudaSuccess ||
             cudaMallocHost(&ls_host, sizeof(molt::LoopState)) != cudaSuccess ||
             cudaMallocHost(&wait_status_host, sizeof(unsigned)) != cudaSuccess)
@@ -911,13 +911,13 @@ struct Solver final : molt_solver {
         }
         double res = INFINITY, tol_used = p.tol, best = INFINITY;
         int k = 0, stall = 0;
-        bool converged = false;
+        bool converged = false, bad = false;   // bad: the last iteration left a NaN (kRedSlots)
         for (k = 1; k <= p.max_iter; ++k) {
-            if ((e = cudaMemsetAsync(red, 0, 2 * sizeof(unsigned long long), st)) != cudaSuccess)
+            if ((e = cudaMemsetAsync(red, 0, molt::kRedSlots * sizeof(unsigned long long), st)) != cudaSuccess)
                 return cuda_fail(e, "memset");
             if ((e = launch_iteration(ps, st)) != cudaSuccess) return cuda_fail(e, "iteration");
-            if ((e = cudaMemcpyAsync(red_host, red, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
-                cudaSuccess)
+            if ((e = cudaMemcpyAsync(red_host, red, molt::kRedSlots * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                     st)) != cudaSuccess)
                 return cuda_fail(e, "residual copy");
             if ((e = cudaMemcpyAsync(wait_status_host, wait_status, sizeof(unsigned), cudaMemcpyDeviceToHost, st)) !=
                 cudaSuccess)
@@ -927,6 +927,7 @@ struct Solver final : molt_solver {
             double dmax, wmax;
             std::memcpy(&dmax, &red_host[0], sizeof(double));
             std::memcpy(&wmax, &red_host[1], sizeof(double));
+            bad = red_host[2] != 0;
             res = dmax;
             if (!std::isfinite(res)) break;
             // FP32 fields cannot resolve changes below a few units in the last place of the
@@ -950,7 +951,8 @@ struct Solver final : molt_solver {
             }
         }
         *iters = converged ? k : std::min(k, p.max_iter);
-        *res_out = res;
+        if (bad) converged = false;
+        *res_out = bad ? NAN : res;
         *tol_out = tol_used;
         return converged ? MOLT_OK : MOLT_ERR_NOT_CONVERGED;
     }
@@ -1213,12 +1215,13 @@ struct Solver final : molt_solver {
                 n_it = std::max({i1.iters[0], i2.iters[0], i3.iters[0]});
             }
             if ((e = molt::max_abs_diff<T>(x, y, static_cast<long long>(count()), red, st)) != cudaSuccess ||
-                (e = cudaMemcpyAsync(red_host, red, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
+                (e = cudaMemcpyAsync(red_host, red, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
                     cudaSuccess ||
                 (e = cudaStreamSynchronize(st)) != cudaSuccess)
                 return cuda_fail(e, "adaptive estimate");
             double diff;
             std::memcpy(&diff, &red_host[0], sizeof(double));
+            if (red_host[1]) diff = NAN;
             const double eta = (sdc || bdf) ? diff : 0.5 * diff;   // the factor 1/2 is Richardson's
             double next;
             const bool ok = step_size_rule(eta, n_it, dt, a, &next, p.max_iter);
@@ -1340,12 +1343,12 @@ struct Solver final : molt_solver {
     double max_diff(const T* a, const T* b, cudaStream_t st, cudaError_t* err) {
         double v = 0.0;
         if ((*err = molt::max_abs_diff<T>(a, b, static_cast<long long>(count()), red, st)) != cudaSuccess ||
-            (*err = cudaMemcpyAsync(red_host, red, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
+            (*err = cudaMemcpyAsync(red_host, red, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
                 cudaSuccess ||
             (*err = cudaStreamSynchronize(st)) != cudaSuccess)
             return 0.0;
         std::memcpy(&v, &red_host[0], sizeof(double));
-        return v;
+        return red_host[1] ? NAN : v;
     }
 
     // Algorithm 1 (Sec. 5) for the vector model, as Sec. 6.2.2 runs it: the Richardson estimate of
@@ -1589,7 +1592,7 @@ struct Solver final : molt_solver {
         }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        cudaMemsetAsync(red, 0, 2 * sizeof(unsigned long long), st);
+        cudaMemsetAsync(red, 0, molt::kRedSlots * sizeof(unsigned long long), st);
         drop_graphs();   // graphs captured the previous choices
         have_prev = have_prev2 = have_sdc = have_adapt_prev = vch_have_prev = vch_adapt_have_prev = false;
         return result;

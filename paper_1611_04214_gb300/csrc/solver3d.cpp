@@ -237,14 +237,16 @@ cudaError_t nest_iteration3(molt_solver3d* s, const molt::StageParams& sp, const
     return molt::nest_rows<float>(lp[0], molt::NEST_ROW_PASS, x, st, nullptr);
 }
 
-double read_max(molt_solver3d* s, const float* a, const float* b, cudaStream_t st, cudaError_t* e) {
+// max |a - b| over the values that are numbers; *bad: whether any was a NaN.
+double read_max(molt_solver3d* s, const float* a, const float* b, cudaStream_t st, cudaError_t* e, bool* bad) {
     double v = 0.0;
     if ((*e = molt::max_abs_diff<float>(a, b, static_cast<long long>(s->n), s->red, st)) != cudaSuccess ||
-        (*e = cudaMemcpyAsync(s->red_host, s->red, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
+        (*e = cudaMemcpyAsync(s->red_host, s->red, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) !=
             cudaSuccess ||
         (*e = cudaStreamSynchronize(st)) != cudaSuccess)
         return 0.0;
     std::memcpy(&v, s->red_host, sizeof(double));
+    *bad = s->red_host[1] != 0;
     s->launches += 1;
     return v;
 }
@@ -283,12 +285,12 @@ molt_status stage3(molt_solver3d* s, double tau, cudaStream_t st, int* iters, do
         return fail3(MOLT_ERR_CUDA, std::string("3D rhs inverse: ") + cudaGetErrorString(e));
     double res = INFINITY, best = INFINITY, tol_used = s->p.tol;
     int k = 0, stall = 0;
-    bool converged = false;
+    bool converged = false, bad = false, bad_max = false;   // bad: the last iteration left a NaN (kRedSlots)
     for (k = 1; k <= s->p.max_iter; ++k) {
         if ((e = iteration3(s, sp, st)) != cudaSuccess)
             return fail3(MOLT_ERR_CUDA, std::string("3D iteration: ") + cudaGetErrorString(e));
-        res = read_max(s, s->wn, s->w, st, &e);
-        const double wmax = e == cudaSuccess ? read_max(s, s->wn, s->zero, st, &e) : 0.0;
+        res = read_max(s, s->wn, s->w, st, &e, &bad);
+        const double wmax = e == cudaSuccess ? read_max(s, s->wn, s->zero, st, &e, &bad_max) : 0.0;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(s->status_host, s->status, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -313,6 +315,7 @@ molt_status stage3(molt_solver3d* s, double tau, cudaStream_t st, int* iters, do
         }
     }
     *iters = converged ? k : std::min(k, s->p.max_iter);
+    if (bad) converged = false, res = NAN;
     *res_out = res;
     *tol_out = tol_used;
     return outcome3(converged, res);
@@ -362,7 +365,7 @@ molt_status molt_solver3d_create(molt_solver3d** out, int nx, int ny, int nz, do
     ok = ok && s->loop.init() && s->alloc(&s->cs.aggL, sc) && s->alloc(&s->cs.aggR, sc) && s->alloc(&s->cs.carL, sc) &&
          s->alloc(&s->cs.carR, sc);
     void* q = nullptr;
-    if (ok && cudaMalloc(&q, 2 * sizeof(unsigned long long)) == cudaSuccess) {
+    if (ok && cudaMalloc(&q, molt::kRedSlots * sizeof(unsigned long long)) == cudaSuccess) {
         s->allocs.push_back(q);
         s->red = static_cast<unsigned long long*>(q);
     } else {

@@ -185,14 +185,13 @@ __device__ __forceinline__ void chunk_finish(T d, int cnt, T cL, T cR, const T (
 // (Sterbenz), and a max is exact in any precision; the block result is widened to FP64.
 template <typename T>
 struct RedAcc {
-    T dmax;   // max |w_new - w|
-    T vmax;   // max |w_new| (stored variable)
+    T dmax;   // max |w_new - w| over numbers (fmax drops a NaN)
+    T vmax;   // max |w_new| (stored variable); a NaN stays (abs_max)
 };
 
-// The larger of a maximum so far and one more absolute value; a NaN stays (fmax would drop it, and an iterate that has
-// overflowed into NaN throughout would leave a residual of zero).  FP64 by unsigned bit patterns: non-negative
-// doubles order like them, a NaN of either sign above infinity (fabs may leave its sign set), and the integer units
-// are idle beside this part's FP64 units.
+// The larger of a maximum so far and one more absolute value; a NaN stays.  FP64 by unsigned bit patterns: non-negative
+// doubles order like them, a NaN of either sign above infinity (fabs may leave its sign set), and the integer
+// units are idle beside this part's FP64 units.
 __device__ __forceinline__ float abs_max(float a, float b) {
     float r;
     asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
@@ -345,7 +344,7 @@ struct OpP4 : OpBase<T> {
     __device__ __forceinline__ void put(int line, int pos, const T (&h)[1], const T (&a)[NA], RedAcc<T>& r) const {
         const T nw = (a[1] + a[0] - a[2]) + h[0];
         w[this->at(line, pos)] = nw;
-        r.dmax = abs_max(r.dmax, fabs(nw - a[0]));
+        r.dmax = fmax(r.dmax, fabs(nw - a[0]));
         r.vmax = abs_max(r.vmax, fabs(nw));
     }
 };
@@ -414,7 +413,7 @@ struct Op1b : OpBase<T> {
     __device__ __forceinline__ void put(int line, int pos, const T (&h)[1], const T (&a)[NA], RedAcc<T>& r) const {
         const T nw = a[1] + h[0];
         w[this->at(line, pos)] = nw;
-        r.dmax = abs_max(r.dmax, fabs(nw - a[0]));
+        r.dmax = fmax(r.dmax, fabs(nw - a[0]));
         r.vmax = abs_max(r.vmax, fabs(nw));
     }
 };
@@ -520,11 +519,13 @@ struct Op1aV : OpBase<T> {
 };
 
 // Block-wide max of the two residual values and one atomic max per block, on the bit patterns
-// (non-negative doubles order like their unsigned bits, a NaN above infinity).
+// (non-negative doubles order like their unsigned bits).  A thread that met a NaN sets the third word instead of
+// its share of max |w_new|: an iterate that has overflowed into NaN throughout would leave a residual of zero.
 template <typename T>
 __device__ __forceinline__ void block_reduce_store(RedAcc<T> r, unsigned long long* slots) {
     __shared__ unsigned long long s_d[32], s_v[32];
-    unsigned long long a = abs_bits(static_cast<double>(r.dmax)), b = abs_bits(static_cast<double>(r.vmax));
+    const bool bad = r.vmax != r.vmax;
+    unsigned long long a = abs_bits(static_cast<double>(r.dmax)), b = bad ? 0ull : abs_bits(static_cast<double>(r.vmax));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         a = max(a, __shfl_xor_sync(kFull, a, o));
@@ -533,6 +534,7 @@ __device__ __forceinline__ void block_reduce_store(RedAcc<T> r, unsigned long lo
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int nthreads = blockDim.x * blockDim.y;
     const int warp = tid >> 5, lane = tid & 31;
+    if (__any_sync(kFull, bad) && lane == 0) atomicMax(&slots[2], 1ull);
     if (lane == 0) {
         s_d[warp] = a;
         s_v[warp] = b;
@@ -631,7 +633,7 @@ struct PipeP4 {
                                              RedAcc<T>& r) const {
         const T nw = (av[1] + av[0] - av[2]) + h[0];
         ov[0] = nw;
-        r.dmax = abs_max(r.dmax, fabs(nw - av[0]));
+        r.dmax = fmax(r.dmax, fabs(nw - av[0]));
         r.vmax = abs_max(r.vmax, fabs(nw));
     }
 };
@@ -668,7 +670,7 @@ struct Pipe1b {
                                              RedAcc<T>& r) const {
         const T nw = av[1] + h[0];
         ov[0] = nw;
-        r.dmax = abs_max(r.dmax, fabs(nw - av[0]));
+        r.dmax = fmax(r.dmax, fabs(nw - av[0]));
         r.vmax = abs_max(r.vmax, fabs(nw));
     }
 };

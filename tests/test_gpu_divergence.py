@@ -1,6 +1,6 @@
-"""GPU: an iteration that overflows ends as not converged, on every path: the residual keeps a NaN (the cubic of an
-overflowing field turns a whole line into NaN within one iteration, so that no finite or infinite value is left beside
-it), and the step reports it instead of a residual of zero."""
+"""GPU: an iteration that overflows ends as not converged, on every path (the cubic of an overflowing field turns a whole
+line into NaN within one iteration, so that no finite or infinite value is left beside it and the residual over
+numbers is zero); independent lines go on beside one that has overflowed."""
 import numpy as np
 import pytest
 
@@ -83,6 +83,26 @@ def test_diverged_sixth_order_lines_are_reported(bc, precision):
         u = torch.full((5, 512), -1.0, device="cuda", dtype=torch.float32 if precision == "fp32" else torch.float64)
         u[2] = _field((1, 512), precision)[0]
         _check(s.step(u, 0.05, raise_on_nonconvergence=False), u)
+
+
+# ... and finish their iterations as they do without it
+@pytest.mark.parametrize("bc", ["periodic", "neumann"])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_lines_go_on_beside_a_diverged_one(bc, precision):
+    from paper_1611_04214_gb300.molt import Fch1D
+    x = torch.linspace(0, 2 * np.pi, 512, dtype=torch.float64)
+    rows = torch.stack([-1 + 0.01 * (k + 1) * torch.cos(x) for k in range(5)])
+    out = []
+    for bad in (False, True):
+        with Fch1D(512, 5, bc=bc, eps=0.18, quad_order=4, tol=1e-30, max_iter=25, precision=precision) as s:
+            u = rows.to(torch.float32 if precision == "fp32" else torch.float64).cuda()
+            if bad:
+                u[2] = _field((1, 512), precision)[0]
+            info = s.step(u, 0.05, raise_on_nonconvergence=False)
+            out.append((u.cpu(), info.iters))
+    assert not torch.isfinite(out[1][0][2]).any() and out[0][1] == out[1][1] == [25]
+    keep = [0, 1, 3, 4]
+    assert torch.equal(out[0][0][keep], out[1][0][keep])
 
 
 @pytest.mark.parametrize("bc", ["periodic", "neumann"])

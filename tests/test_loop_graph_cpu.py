@@ -65,27 +65,32 @@ cudaError_t loop_check(cudaGraphConditionalHandle, LoopState*, unsigned long lon
 }  // namespace molt
 
 int main() {
-    struct Case { const char* name; double res[12]; int n; bool fp32; double tol; int max_iter; };
+    // residuals over numbers; from iteration `bad` on (counted from 1, 0: never) one value is a NaN
+    struct Case { const char* name; double res[12]; int n; bool fp32; double tol; int max_iter; int bad; };
     const double u = 5.9604644775390625e-08;   // 2^-24, max|w| = 1
     const Case cases[] = {
         {"converges", {1, 0.1, 0.01, 1e-9}, 4, false, 1e-6, 50},
         {"floor", {1, 0.1, 1.5 * u}, 3, true, 1e-30, 50},
         {"cap", {1, 0.5, 0.25, 0.125}, 4, false, 1e-6, 4},
         {"stall", {30 * u, 31 * u, 31 * u, 31 * u, 31 * u, 31 * u, 31 * u}, 7, true, 1e-30, 50},
-        {"overflow", {1, 1e20, NAN}, 3, false, 1e-6, 50},
+        {"overflow", {1, 1e20, INFINITY}, 3, false, 1e-6, 50},
+        {"nan", {1, 1e20, 0}, 3, false, 1e-6, 50, 3},
+        {"others", {1, 0.1, 0.01, 1e-3, 1e-9}, 5, false, 1e-6, 50, 2},
+        {"nancap", {1, 0.5, 0.25, 0.125}, 4, false, 1e-6, 4, 4},
     };
     for (fail = 1; fail <= 6; ++fail)
         for (const Case& c : cases) {
             molt::LoopGraphs loop;
             if (!loop.init()) return 1;
-            unsigned long long red[2] = {7, 7};
+            unsigned long long red[molt::kRedSlots] = {7, 7, 7};
             int k = 0;
             auto body = [&](cudaStream_t s) {
                 if (s == kUser) {
-                    if (red[0] || red[1] || k >= c.n) return cudaErrorUnknown;   // slots cleared, no iteration too many
+                    if (red[0] || red[1] || red[2] || k >= c.n) return cudaErrorUnknown;   // slots cleared, no iteration too many
                     const double r = c.res[k++], w = 1.0;
                     std::memcpy(&red[0], &r, 8);
                     std::memcpy(&red[1], &w, 8);
+                    red[2] = c.bad && k >= c.bad ? 1 : 0;
                 }
                 return cudaSuccess;
             };
@@ -118,4 +123,8 @@ def test_host_runs_the_loop_where_a_graph_call_fails(outcomes, call):
     assert outcomes[call, "cap"] == (0, 4, 0, 0.125, 1e-6, 1)
     assert outcomes[call, "stall"] == (0, 7, 1, 31 * u, 31 * u, 1)
     e, k, conv, res, _, _ = outcomes[call, "overflow"]
-    assert (e, k, conv) == (0, 3, 0) and math.isnan(res)
+    assert (e, k, conv) == (0, 3, 0) and math.isinf(res)
+    # a NaN: the iteration ends when what is left of the residual does, never as converged
+    for name, its in (("nan", 3), ("others", 5), ("nancap", 4)):
+        e, k, conv, res, _, _ = outcomes[call, name]
+        assert (e, k, conv) == (0, its, 0) and math.isnan(res), name
