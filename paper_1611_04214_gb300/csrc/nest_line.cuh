@@ -162,12 +162,12 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
         for (int k = 0; k < K; ++k)
             if (k < cnt) {
                 const T nw = y[k] + out[k];
-                dm = fmax(dm, fabs(nw - w[k]));
+                dm = abs_max(dm, fabs(nw - w[k]));
                 vm = abs_max(vm, fabs(nw));
                 w[k] = a.fix && (start + k == 0 || start + k == n - 1) ? a.wall : nw;
             }
-        const bool nan_here = vm != vm;
-        dm = nest_warp_max(dm);
+        const bool nan_here = vm != vm || dm != dm;   // (the line is NaN throughout then: nest_reduce)
+        dm = nest_warp_max(nan_here ? T(0) : dm);
         vm = nest_warp_max(nan_here ? T(0) : vm);
         if (g.c.lane == 0) {
             s_max[0][g.c.warp] = dm;
@@ -178,8 +178,8 @@ nest_line_kernel(const __grid_constant__ LineParams<typename N::T> li, const __g
             // as loop_check: tolerance, FP32 floor of 2 ulp of max|w|, stall at the FP32 noise floor, cap, NaN
             T d = T(0), v = T(0);
             for (int q = 0; q < g.c.nwarps; ++q) {
-                d = fmax(d, s_max[0][q]);
-                v = fmax(v, s_max[1][q]);
+                d = abs_max(d, s_max[0][q]);
+                v = abs_max(v, s_max[1][q]);
             }
             res = static_cast<double>(d);
             vmax = static_cast<double>(v);

@@ -214,7 +214,9 @@ __device__ __forceinline__ void nest_row_load(const typename N::T* f, int half, 
 }
 
 // Block maximum of the residual values into the FP64 slots; blocks that would not raise a slot leave
-// it alone (the slots only grow, so a stale read costs an atomic at most).  NaN as in block_reduce_store.
+// it alone (the slots only grow, so a stale read costs an atomic at most).  A NaN marks the third slot, as in
+// block_reduce_store; a thread's nodes belong to one line, which is NaN throughout then, so the thread's whole share is
+// left out.
 template <typename T>
 __device__ __forceinline__ T nest_warp_max(T v) {
     if constexpr (sizeof(T) == 4) {
@@ -222,15 +224,15 @@ __device__ __forceinline__ T nest_warp_max(T v) {
         return __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(v)));
     } else {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(kFull, v, o));
+        for (int o = 16; o > 0; o >>= 1) v = abs_max(v, __shfl_xor_sync(kFull, v, o));
         return v;
     }
 }
 template <typename T>
 __device__ __forceinline__ void nest_reduce(RedAcc<T> r, unsigned long long* slots) {
     __shared__ T s_max[2][16];
-    const bool bad = r.vmax != r.vmax;
-    const T dm = nest_warp_max(r.dmax), vm = nest_warp_max(bad ? T(0) : r.vmax);
+    const bool bad = r.vmax != r.vmax || r.dmax != r.dmax;
+    const T dm = nest_warp_max(bad ? T(0) : r.dmax), vm = nest_warp_max(bad ? T(0) : r.vmax);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (__any_sync(kFull, bad) && lane == 0) atomicMax(slots + 2, 1ull);
     if (lane == 0) {
@@ -240,7 +242,7 @@ __device__ __forceinline__ void nest_reduce(RedAcc<T> r, unsigned long long* slo
     __syncthreads();
     if (threadIdx.x < 2) {
         T m = T(0);
-        for (int w = 0; w < nw; ++w) m = fmax(m, s_max[threadIdx.x][w]);
+        for (int w = 0; w < nw; ++w) m = abs_max(m, s_max[threadIdx.x][w]);
         const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(static_cast<double>(m)));
         if (b > *static_cast<volatile unsigned long long*>(slots + threadIdx.x)) atomicMax(slots + threadIdx.x, b);
     }
@@ -422,7 +424,7 @@ nest_rows_kernel(const __grid_constant__ LineParams<typename N::T> lp,
         const bool wall_row = a.fix && (line == 0 || line == a.nlines - 1);
         auto put = [&](T h, T e, T o, int p) {
             const T nw = o + (e + h);
-            red.dmax = fmax(red.dmax, fabs(nw - o));
+            red.dmax = abs_max(red.dmax, fabs(nw - o));
             red.vmax = abs_max(red.vmax, fabs(nw));
             return a.fix && (wall_row || p == 0 || p == lp.n - 1) ? a.wall : nw;
         };
@@ -533,7 +535,7 @@ nest_fch_kernel(const __grid_constant__ LineParams<typename N::T> lp,
                 const V e = N::fma(m1, x[H + k], out[k]);
 #pragma unroll
                 for (int q = 0; q < N::W; ++q) {
-                    red.dmax = fmax(red.dmax, fabs(N::get(e, q)));
+                    red.dmax = abs_max(red.dmax, fabs(N::get(e, q)));
                     red.vmax = abs_max(red.vmax, fabs(N::get(out[k], q)));
                 }
             }
@@ -617,7 +619,7 @@ nest_fch2_kernel(const __grid_constant__ LineParams<typename N::T> lp,
                     const V e = N::fma(m1, o[i], out[4 * j + i]);
 #pragma unroll
                     for (int q = 0; q < N::W; ++q) {
-                        red.dmax = fmax(red.dmax, fabs(N::get(e, q)));
+                        red.dmax = abs_max(red.dmax, fabs(N::get(e, q)));
                         red.vmax = abs_max(red.vmax, fabs(N::get(out[4 * j + i], q)));
                     }
                 }

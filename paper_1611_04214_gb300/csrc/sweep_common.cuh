@@ -185,7 +185,7 @@ __device__ __forceinline__ void chunk_finish(T d, int cnt, T cL, T cR, const T (
 // (Sterbenz), and a max is exact in any precision; the block result is widened to FP64.
 template <typename T>
 struct RedAcc {
-    T dmax;   // max |w_new - w| over numbers (fmax drops a NaN)
+    T dmax;   // max |w_new - w| over numbers (fmax drops a NaN; see nest_reduce for threads of one line)
     T vmax;   // max |w_new| (stored variable); a NaN stays (abs_max)
 };
 
