@@ -39,7 +39,7 @@ extern "C" {
 typedef enum {
     MOLT_OK = 0,
     MOLT_ERR_ARG = -1,            /* bad size, parameter or pointer */
-    MOLT_ERR_NOT_CONVERGED = -2,  /* a stage hit max_iter; the field holds the last iterate */
+    MOLT_ERR_NOT_CONVERGED = -2,  /* a stage hit max_iter or overflowed; the field holds the last iterate */
     MOLT_ERR_CUDA = -3,           /* a CUDA runtime call failed */
     MOLT_ERR_OOM = -4,            /* device workspace could not be allocated */
     MOLT_ERR_UNSUPPORTED = -5     /* valid request this build does not implement */
@@ -128,9 +128,10 @@ molt_status molt_reset_history(molt_solver* solver);
  * (w = u on periodic/Neumann grids, w = u + 1 on Dirichlet grids), so for FP32 solvers the
  * tolerance applied is max(tol, 2 * 2^-24 * max|w|), and an iteration whose residual is below
  * 64 * 2^-24 * max|w| and has not reached a new minimum for 6 iterations is accepted as
- * converged at FP32 precision (the rounding noise floor); `info->tol_used` reports the tolerance (or residual) that ended the stage.  BDF2 and SDC2 keep history between calls made
- * with the same dt.  Returns MOLT_ERR_NOT_CONVERGED (field = last iterate, history
- * updated) when a stage hits max_iter; `info` may be NULL. */
+ * converged at FP32 precision (the rounding noise floor); `info->tol_used` reports the tolerance (or residual) that ended
+ * the stage.  BDF2 and SDC2 keep history between calls made with the same dt.  Returns
+ * MOLT_ERR_NOT_CONVERGED (field = last iterate, history updated) when a stage hits max_iter or leaves a NaN or
+ * an infinity (the residual is then not finite; so for every step of this header); `info` may be NULL. */
 molt_status molt_step(molt_solver* solver, void* u_dev, double dt, int scheme, void* stream,
                       molt_step_info* info);
 
@@ -416,7 +417,7 @@ molt_status molt_batch_set_schedule(molt_batch* batch, int grid_rows, int grid_c
  * CH_2D_Doperator1); the 2D fixed-point iteration of Sec. 5.1 then holds with X in place of
  * D_x D_y.  FP32 fields of nz * ny * nx floats, row-major with x fastest, periodic or Neumann
  * lines (the grid conventions of molt_grid_create per axis).  With equal factors an iteration is one
- * pass per axis, its loop on the device; with different factors, or lines that those passes do not
+ * pass per axis, its loop on the device (driven by the host where no graph can be built); with different factors, or lines that those passes do not
  * take, it is a sequence of single line sweeps over the whole field.  Errors of these calls are
  * reported by molt_last_error(NULL). */
 typedef struct molt_solver3d molt_solver3d;
