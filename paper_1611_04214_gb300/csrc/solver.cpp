@@ -576,9 +576,10 @@ struct Solver final : molt_solver {
     //   FP64: every size (1024^2 510 / 309, 2048^2 1777 / 1072, 8192^2 29800 / 22000; columns over clusters of 13 to 16 blocks
     //   gain least, 300 x 7000 1379 / 1119, 1024 x 8192 3841 / 2758).
     //   FP32: from 256 nodes a side (shorter lines run the block bodies of the batched path, which a single grid with
-    //   rows below 1024 and columns below 256 matches bit for bit; longer lines beside a short side were not measured); 1024^2 periodic / Neumann 46 / 25 and 60 / 28, 2048^2 92 / 77 and
-    //   128 / 78, 4096^2 282 / 272 and 318 / 273, 5000 x 7001 1675 / 1013 and 1732 / 1015, 512 x 8192 143 / 92.  Columns
-    //   of more than 6144 nodes are spread over clusters of 13 to 16 blocks, few of which fit at a time: where the
+    //   rows below 1024 and columns below 256 matches bit for bit; longer lines beside a short side were not
+    //   measured); 1024^2 periodic / Neumann 46 / 25 and 60 / 28, 2048^2 92 / 77 and 128 / 78, 4096^2 282 / 272 and
+    //   318 / 273, 5000 x 7001 1675 / 1013 and 1732 / 1015, 512 x 8192 143 / 92.  Columns of more than 6144 nodes are
+    //   spread over clusters of 13 to 16 blocks, few of which fit at a time: where the
     //   rows suit the pipelined kernel of the four passes (whole warps of 16-node chunks from 1024 nodes), those stay,
     //   2048 x 8192 272 / 325 and 288 / 326, 8192^2 1035 / 1279 and 1072 / 1282; but 1024 x 6000 133 / 117,
     //   4096 x 6000 409 / 412 and 425 / 415.  Vector model: 4096^2 767 / 590, 2048 x 8192 680 / 697.
